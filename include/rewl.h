@@ -96,11 +96,12 @@ typedef struct {
   int32_t profile;               /* 1 = time every sweep launch with CUDA events on the solve's stream
                                     (plain mode); read back through rewl_info */
   int32_t sweep_variant;         /* sweep kernel form, identical results: REWL_SWEEP_AUTO (default: the
-                                    ring form when the solve has at most 8 walkers per SM and lanes / walkers
-                                    per block are not forced, else the chain form), REWL_SWEEP_CHAIN
-                                    (two-deep chain), REWL_SWEEP_STAGED (staged one-deep chain),
-                                    REWL_SWEEP_RING (the chain with its draws made by a second, producer warp
-                                    of the CTA; 32 lanes and one walker per CTA) */
+                                    ring form when its CTAs, one a walker, run in one wave (7 per SM; fewer for
+                                    wide windows) and lanes / walkers per block are not forced, else the chain
+                                    form), REWL_SWEEP_CHAIN (32 lanes: the warp decides 32 trials together and
+                                    makes its own draws; fewer lanes: two-deep chain), REWL_SWEEP_STAGED (staged
+                                    one-deep chain), REWL_SWEEP_RING (32 trials decided together, draws made by
+                                    producer warps of the CTA; 32 lanes and one walker per CTA) */
   int32_t prefetch_draws;        /* 1 = in plain mode with variant 0 the draws of the next block (sites,
                                     ln u, conflict masks) are prepared on a second stream while the current
                                     block runs, when both buffers fit in 1 GiB; 0 = no (default: kernels

@@ -610,20 +610,9 @@ __device__ __noinline__ bool exact_accept_fx(const DevState& S, const Problem& P
 }
 
 // ---------------------------------------------------------------------------
-// Warp-specialised form (variant kSweepRing): a producer warp computes the
-// draws of upcoming groups (Philox, site, Potts offset, ln u, conflict mask)
-// into a ring of kRingSlots groups in shared memory while the walker's warp
-// runs the sequential chain; the walker's warp only evaluates the moves on the
-// current configuration.  The two warps sit on different SM sub-partitions,
-// so the producer does not take issue slots from the chain.  Hand-off through
-// mbarriers: full[s] (32 producer arrivals) and empty[s] (32 walker-warp
-// arrivals); every wait is bounded by a clock deadline, after which the warp
+// mbarriers of the ring form (rewl_resolve.cuh); every wait is bounded by a clock deadline, after which the warp
 // records an error (DevState.error) and leaves its loop.
 // ---------------------------------------------------------------------------
-constexpr int kRingSlots = 4;
-// the ring, its full and empty barriers, and one 16-byte word that says which warp is the walker's
-constexpr size_t kRingBytes = (size_t)kRingSlots * 32 * sizeof(PreTrial) + 2 * kRingSlots * sizeof(uint64_t) + 16;
-
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);
 }
@@ -655,41 +644,19 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, l
   }
 }
 
-// The draw of trial t of walker W, with the conflict mask of its group of 32
-// (lane = t mod 32); the same values the in-kernel path computes.
-template <int MODEL>
-__device__ __forceinline__ PreTrial make_pretrial(const Problem& P, uint64_t t, int W, int lane) {
-  const U4 r = philox10((uint32_t)t, (uint32_t)(t >> 32), (uint32_t)W, kTagFlip, P.seed_lo, P.seed_hi);
-  int x, y;
-  uint32_t pv;
-  trial_site<MODEL>(P, r, x, y, pv);
-  const float uf = __ull2float_rn(2ull * u52_bits(r.z, r.w) + 1ull) * 0x1p-53f;
-  const int64_t thr = __float2ll_rn(logf(uf) * 1099511627776.0f);
-  const uint32_t M = conflict_mask<MODEL, 32>(P, x, y, pv, lane, 0xffffffffu);
-  return PreTrial{(uint32_t)x | ((uint32_t)y << 8) | (pv << 16), M, thr};
-}
-
 // Runs the sweeps of the nloc walkers wids[0..nloc) of one CTA (wpb walkers per CTA).
-// RING: warp-specialised form (G = 32, one walker, 64 threads: one warp the
-// walker, the other the producer of its draws).
-template <int MODEL, int G, bool RING = false>
+template <int MODEL, int G>
 __device__ __forceinline__ void sweep_chain_body(const Problem& P, const DevState& S, uint32_t n_att, int wpb,
                                                  const int32_t* wids, int nloc, const PreTrial* pre = nullptr,
-                                                 uint32_t pre_stride = 0,
-                                                 long long wait_cycles = kDefaultWaitCycles) {
+                                                 uint32_t pre_stride = 0) {
   static_assert(G == 1 || G == 2 || G == 4 || G == 8 || G == 16 || G == 32, "G");
-  static_assert(!RING || G == 32, "the ring form runs one walker on one warp");
   // The sequential step skips the trials it need not visit (accepted for sure, energy unchanged)
   // when one walker owns the warp; with several walkers per warp the chains run in lockstep, the
   // longest decides, and the skip would cost more than it saves.
   constexpr bool kSkip = G == 32;
   extern __shared__ __align__(16) unsigned char smem[];
   const int wpad = P.w + 2 * kGuardBins;
-  PreTrial* s_ring = reinterpret_cast<PreTrial*>(smem);                                  // [kRingSlots][32]
-  uint64_t* s_full = reinterpret_cast<uint64_t*>(s_ring + kRingSlots * 32);              // [kRingSlots]
-  uint64_t* s_empty = s_full + kRingSlots;                                               // [kRingSlots]
-  int* s_swap = reinterpret_cast<int*>(s_empty + kRingSlots);                             // RING: 1 = roles swapped
-  HotTrial* s_hot = reinterpret_cast<HotTrial*>(smem + (RING ? kRingBytes : 0));         // [G][wpb]
+  HotTrial* s_hot = reinterpret_cast<HotTrial*>(smem);                                    // [G][wpb]
   ColdTrial* s_cold = reinterpret_cast<ColdTrial*>(s_hot + (G > 1 ? (size_t)wpb * G : 0));  // [G][wpb]
   int64_t* s_fx = reinterpret_cast<int64_t*>(s_cold + (G > 1 ? (size_t)wpb * G : 0));      // [wpad][wpb]
   uint32_t* s_lat = reinterpret_cast<uint32_t*>(s_fx + (size_t)wpad * wpb);
@@ -709,51 +676,10 @@ __device__ __forceinline__ void sweep_chain_body(const Problem& P, const DevStat
   }
   if (MODEL == kEA || MODEL == kEA3)
     for (int i = tid; i < P.j_words; i += nthr) s_J[i] = S.J[i];
-  // RING: which warp of the CTA is the walker's.  An SM spreads its warps over its four
-  // sub-partitions by hardware slot (%warpid mod 4), and a CTA of two warps takes two neighbouring
-  // slots, so with several CTAs on one SM the first warps of all of them share the even
-  // sub-partitions.  A CTA whose first slot lies in an odd group of four gives the walker to its
-  // second warp, which spreads the chains over all four.  Only the placement depends on it: the
-  // two roles compute the same whichever warp takes them.  rtid is the thread's index in its
-  // role: [0, 32) the walker's warp, [32, 64) the producer.
-  int rtid = tid;
-  if constexpr (RING) {
-    if (tid == 0) {
-      uint32_t slot;
-      asm volatile("mov.u32 %0, %%warpid;" : "=r"(slot));
-      *s_swap = (int)((slot >> 2) & 1u);
-      for (int k = 0; k < kRingSlots; ++k) {
-        mbar_init(&s_full[k], 32);
-        mbar_init(&s_empty[k], 32);
-      }
-    }
-    __syncthreads();
-    if (*s_swap) rtid = tid ^ 32;
-  } else {
-    __syncthreads();
-  }
+  __syncthreads();
 
-  if (RING && rtid >= 32) {  // ---- producer warp
-    if (nloc > 0) {
-      const int W = wids[0];
-      const uint64_t t0 = S.clock[0] * (uint64_t)P.N;
-      const int lane = rtid - 32;
-      const uint32_t n_groups = (n_att + 31) / 32;
-      const long long deadline = __shfl_sync(0xffffffffu, clock64(), 0) + wait_cycles;
-      for (uint32_t g = 0; g < n_groups; ++g) {
-        const uint32_t sl = g % kRingSlots, rnd = g / kRingSlots;
-        if (rnd >= 1 && !mbar_wait_warp(&s_empty[sl], (rnd - 1) & 1u, deadline)) {
-          if (lane == 0) atomicOr(S.error, 1);
-          break;
-        }
-        s_ring[sl * 32 + lane] = make_pretrial<MODEL>(P, t0 + (uint64_t)g * 32 + lane, W, lane);
-        mbar_arrive(&s_full[sl]);
-      }
-    }
-  }
-
-  const int lw = rtid / G, lane = rtid % G;
-  bool valid = lw < nloc && !(RING && rtid >= 32);
+  const int lw = tid / G, lane = tid % G;
+  bool valid = lw < nloc;
   int W = 0, a = 0, bin = 0, kexp = 0, wstart = 0;
   if (valid) {
     W = wids[lw];
@@ -780,8 +706,6 @@ __device__ __forceinline__ void sweep_chain_body(const Problem& P, const DevStat
     const PreTrial* my_pre = pre ? pre + (size_t)W * pre_stride : nullptr;
     PreTrial nxt_pre{0u, 0u, 0};
     if (my_pre && (uint32_t)lane < n_att) nxt_pre = my_pre[lane];
-    long long deadline = 0;
-    if constexpr (RING) deadline = __shfl_sync(0xffffffffu, clock64(), 0) + wait_cycles;
     const int lsh = kFxBits - kexp;  // ln f = 2^-kexp is 2^lsh shadow units
     const int64_t lnf_fx = 1ll << lsh;
     for (uint32_t base = 0; base < n_att; base += G) {
@@ -791,20 +715,7 @@ __device__ __forceinline__ void sweep_chain_body(const Problem& P, const DevStat
       {
         int x, y;
         uint32_t pv, M = 0;
-        if constexpr (RING) {  // draw from the producer warp's ring
-          const uint32_t g = base / 32, sl = g % kRingSlots;
-          if (!mbar_wait_warp(&s_full[sl], (g / kRingSlots) & 1u, deadline)) {
-            if (lane == 0) atomicOr(S.error, 2);
-            break;  // uniform over the warp: every lane waits on the same phase
-          }
-          const PreTrial pt = s_ring[sl * 32 + lane];
-          mbar_arrive(&s_empty[sl]);
-          x = (int)(pt.pk & 0xffu);
-          y = (int)((pt.pk >> 8) & 0xffu);
-          pv = pt.pk >> 16;
-          M = pt.mask;
-          tr.thr = pt.thr;
-        } else if (my_pre) {  // draw prepared ahead by k_precompute; prefetch the next group's
+        if (my_pre) {  // draw prepared ahead by k_precompute; prefetch the next group's
           const PreTrial pt = nxt_pre;
           if (base + G + (uint32_t)lane < n_att) nxt_pre = my_pre[base + G + lane];
           x = (int)(pt.pk & 0xffu);
@@ -998,17 +909,31 @@ __device__ __forceinline__ void sweep_chain_body(const Problem& P, const DevStat
   }
 }
 
+}  // namespace rewl
+#include "rewl_resolve.cuh"
+namespace rewl {
+
+// wpb walkers a CTA, one warp each, every group of 32 trials decided together.  Bound by issue (72% of the
+// active cycles, the integer pipe 69%): 24 warps an SM at 80 registers; 64 registers for 32 warps spill and lose 6%.
+constexpr int kResolveWarps = 2;  // most walkers a CTA: they share nothing but the couplings
+template <int MODEL>
+__global__ void __launch_bounds__(32 * kResolveWarps, 12) k_sweep_resolve(Problem P, DevState S, SweepLaunch A) {
+  const int first = blockIdx.x * A.wpb;
+  sweep_resolve_body<MODEL>(P, S, A.n_att, S.active + first, min(A.wpb, A.n_active - first));
+}
+
+// One walker a CTA, its draws made by further warps.
+constexpr int kRingCtas = 7;  // that an SM's registers hold (97 a thread)
+template <int MODEL>
+__global__ void __launch_bounds__(kRingThreads, kRingCtas) k_sweep_resolve_ring(Problem P, DevState S, SweepLaunch A) {
+  sweep_resolve_ring_body<MODEL>(P, S, A.n_att, S.active[blockIdx.x], A.wait_cycles);
+}
+
 template <int MODEL, int G>
 __global__ void __launch_bounds__(256, 1) k_sweep_chain(Problem P, DevState S, SweepLaunch A) {
   const int first = blockIdx.x * A.wpb;
   sweep_chain_body<MODEL, G>(P, S, A.n_att, A.wpb, S.active + first, min(A.wpb, A.n_active - first), A.pre,
                              A.pre_stride);
-}
-
-// One walker per CTA of 64 threads (G = 32): one warp the walker, the other its draws.
-template <int MODEL>
-__global__ void __launch_bounds__(64, 1) k_sweep_ring(Problem P, DevState S, SweepLaunch A) {
-  sweep_chain_body<MODEL, 32, true>(P, S, A.n_att, 1, S.active + blockIdx.x, 1, nullptr, 0, A.wait_cycles);
 }
 
 // ---------------------------------------------------------------------------
@@ -1243,7 +1168,8 @@ __global__ void k_flat_merge(Problem P, DevState S) { flat_merge_body(P, S, (int
 // own schedule, streams and state, so its trajectory is the one it has alone.
 // ---------------------------------------------------------------------------
 // A shape group holds one model, so each form is instantiated per model and
-// the group's launch picks the one of its model.  One walker per 32-lane CTA:
+// the group's launch picks the one of its model.  The chain form, one walker per 32-lane CTA, for
+// windows that only fit it:
 template <int MODEL>
 __global__ void __launch_bounds__(32, 16) k_sweep_batch(const BatchSlot* __restrict__ slots,
                                                         const BatchWalker* __restrict__ list) {
@@ -1258,46 +1184,18 @@ __global__ void __launch_bounds__(32, 16) k_sweep_batch(const BatchSlot* __restr
   sweep_chain_body<MODEL, 32>(P, S, n_att, 1, &wid, 1);
 }
 
-// The same with a producer warp per walker (the ring form): for rounds with few
-// walkers on the GPU, where each walker's chain has an SM sub-partition of its own.
-template <int MODEL>
-__global__ void __launch_bounds__(64, 8) k_sweep_batch_ring(const BatchSlot* __restrict__ slots,
-                                                            const BatchWalker* __restrict__ list) {
-  __shared__ int32_t wid;
+// The forms that decide 32 trials together, one walker per CTA: with producer warps for rounds with few walkers on
+// the GPU (each walker's passes are latency-bound), without for rounds with many (the issue slots are what runs out).
+template <int MODEL, bool RING>
+__global__ void __launch_bounds__(RING ? kRingThreads : 32, RING ? kRingCtas : 16) k_sweep_batch_resolve(
+    const BatchSlot* __restrict__ slots, const BatchWalker* __restrict__ list) {
   const BatchWalker bw = list[blockIdx.x];
   const Problem P = slots[bw.slot].P;
   const DevState S = slots[bw.slot].S;
   const uint32_t n_att = slots[bw.slot].n_att;
   if (!slots[bw.slot].active || S.done[bw.W / P.m]) return;  // uniform over the CTA
-  if (threadIdx.x == 0) wid = bw.W;
-  __syncthreads();
-  sweep_chain_body<MODEL, 32, true>(P, S, n_att, 1, &wid, 1);
-}
-
-// For rounds with many walkers on the GPU (the chains share the SMs and the
-// issue slots are what runs out): up to 4 walkers of one request per CTA, 8
-// lanes each, so that one instruction of the sequential step serves 4 chains.
-// Entry (slot, W0) covers walkers W0 .. W0+3 of the slot; walkers of finished
-// windows are left out.
-template <int MODEL>
-__global__ void __launch_bounds__(32, 16) k_sweep_batch_quad(const BatchSlot* __restrict__ slots,
-                                                             const BatchWalker* __restrict__ list) {
-  __shared__ int32_t wids[4];
-  __shared__ int32_t nloc;
-  const BatchWalker bw = list[blockIdx.x];
-  const Problem P = slots[bw.slot].P;
-  const DevState S = slots[bw.slot].S;
-  const uint32_t n_att = slots[bw.slot].n_att;
-  if (!slots[bw.slot].active) return;  // uniform over the CTA
-  if (threadIdx.x == 0) {
-    int n = 0;
-    for (int W = bw.W; W < bw.W + 4 && W < P.n_walkers; ++W)
-      if (!S.done[W / P.m]) wids[n++] = W;
-    nloc = n;
-  }
-  __syncthreads();
-  if (nloc == 0) return;  // uniform over the CTA
-  sweep_chain_body<MODEL, 8>(P, S, n_att, 4, wids, nloc);
+  if constexpr (RING) sweep_resolve_ring_body<MODEL>(P, S, n_att, bw.W, kDefaultWaitCycles);
+  else sweep_resolve_body<MODEL>(P, S, n_att, &bw.W, 1);
 }
 
 __global__ void k_exchange_batch(const BatchSlot* __restrict__ slots, int max_pairs) {
@@ -1344,16 +1242,15 @@ __global__ void k_slot_report(const BatchSlot* __restrict__ slots, int n_slots, 
 // allowance stays below the 227 KB per-CTA limit.
 constexpr int kBatchDynSmem = 226 * 1024;
 
-size_t ring_extra_smem() { return kRingBytes; }
 size_t batch_smem_limit() { return kBatchDynSmem; }
 
 template <int MODEL>
 static cudaError_t prepare_sweep_batch_m() {
   cudaError_t e = cudaFuncSetAttribute(k_sweep_batch<MODEL>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBatchDynSmem);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_sweep_batch_quad<MODEL>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBatchDynSmem);
+  e = cudaFuncSetAttribute(k_sweep_batch_resolve<MODEL, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBatchDynSmem);
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_sweep_batch_ring<MODEL>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBatchDynSmem);
+  return cudaFuncSetAttribute(k_sweep_batch_resolve<MODEL, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBatchDynSmem);
 }
 
 cudaError_t prepare_sweep_batch() {
@@ -1367,8 +1264,8 @@ cudaError_t prepare_sweep_batch() {
 template <int MODEL>
 static void launch_sweep_batch_m(const BatchSlot* d_slots, const BatchWalker* d_list, int n_list, size_t smem,
                                  int form, cudaStream_t st) {
-  if (form == kBatchRing) k_sweep_batch_ring<MODEL><<<n_list, 64, smem + kRingBytes, st>>>(d_slots, d_list);
-  else if (form == kBatchQuad) k_sweep_batch_quad<MODEL><<<n_list, 32, smem, st>>>(d_slots, d_list);
+  if (form == kBatchRing) k_sweep_batch_resolve<MODEL, true><<<n_list, kRingThreads, smem, st>>>(d_slots, d_list);
+  else if (form == kBatchOne) k_sweep_batch_resolve<MODEL, false><<<n_list, 32, smem, st>>>(d_slots, d_list);
   else k_sweep_batch<MODEL><<<n_list, 32, smem, st>>>(d_slots, d_list);
 }
 
@@ -1404,7 +1301,21 @@ cudaError_t launch_slot_report(const BatchSlot* d_slots, int n_slots, SlotReport
 // ---------------------------------------------------------------------------
 // Launch wrappers
 // ---------------------------------------------------------------------------
-// G <= 4 lanes per walker: k_sweep; G >= 8: the speculative k_sweep_spec.
+constexpr size_t kMaxSmem = 227 * 1024;
+
+// Whether a whole-warp solve (32 lanes a walker, no prepared draws) runs the forms that decide 32 trials
+// together: always, unless their tables push a very wide window past the shared memory that the chain form,
+// about 1 KB smaller, still fits in.
+bool resolve_fits(const Problem& P, int wpb) { return resolve_smem_bytes(P, wpb, false) <= kMaxSmem; }
+size_t resolve_smem(const Problem& P, int wpb, bool ring) { return resolve_smem_bytes(P, wpb, ring); }
+
+// Walkers an SM runs at once in the ring form.  Up to there the ring form is the faster one (Ising 32 x 32, ln f =
+// 2^-18, 1024 walkers: 64 cycles a trial against 76 with the draws in the same warp; 64 walkers: 41 against 59);
+// a second wave of CTAs would double its time (1280 walkers of Ising 21 x 21: 97 against 90).
+int ring_walkers_per_sm(const Problem& P) {
+  return (int)std::min<size_t>(kRingCtas, kMaxSmem / (resolve_smem_bytes(P, 1, true) + 1024));
+}
+
 template <int MODEL, int G>
 static auto sweep_kernel(int variant) {
   return variant == kSweepStaged ? k_sweep_spec<MODEL, G> : k_sweep_chain<MODEL, G>;
@@ -1412,13 +1323,15 @@ static auto sweep_kernel(int variant) {
 
 template <int MODEL, int G>
 static cudaError_t prepare_sweep_t() {
-  cudaError_t e = cudaFuncSetAttribute(k_sweep_spec<MODEL, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+  cudaError_t e = cudaFuncSetAttribute(k_sweep_spec<MODEL, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
   if (e != cudaSuccess) return e;
   if (G == 32) {
-    e = cudaFuncSetAttribute(k_sweep_ring<MODEL>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    e = cudaFuncSetAttribute(k_sweep_resolve_ring<MODEL>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_sweep_resolve<MODEL>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
     if (e != cudaSuccess) return e;
   }
-  return cudaFuncSetAttribute(k_sweep_chain<MODEL, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+  return cudaFuncSetAttribute(k_sweep_chain<MODEL, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
 }
 
 template <int MODEL>
@@ -1448,12 +1361,22 @@ cudaError_t prepare_sweep(int G, int model) {
 template <int MODEL, int G>
 static cudaError_t launch_sweep_t(const Problem& P, const DevState& S, const SweepLaunch& A, size_t smem,
                                   cudaStream_t st) {
-  if (A.variant == kSweepRing) {  // one walker per CTA: its warp and a producer warp
-    if (G != 32 || A.wpb != 1) return cudaErrorInvalidValue;
-    k_sweep_ring<MODEL><<<A.n_active, 64, smem, st>>>(P, S, A);
-    return cudaGetLastError();
-  }
   const int blocks = (A.n_active + A.wpb - 1) / A.wpb;
+  if (A.variant == kSweepRing && (G != 32 || A.wpb != 1)) return cudaErrorInvalidValue;
+  if (G == 32 && A.variant != kSweepStaged && !A.pre) {
+    const size_t ring = resolve_smem_bytes(P, 1, true);
+    if (A.variant == kSweepRing && ring <= kMaxSmem) {
+      k_sweep_resolve_ring<MODEL><<<A.n_active, kRingThreads, ring, st>>>(P, S, A);
+      return cudaGetLastError();
+    }
+    SweepLaunch B = A;
+    B.wpb = std::min(A.wpb, kResolveWarps);
+    if (B.wpb > 1 && !resolve_fits(P, B.wpb)) B.wpb = 1;
+    if (resolve_fits(P, B.wpb)) {
+      k_sweep_resolve<MODEL><<<(A.n_active + B.wpb - 1) / B.wpb, B.wpb * 32, resolve_smem_bytes(P, B.wpb, false), st>>>(P, S, B);
+      return cudaGetLastError();
+    }
+  }
   sweep_kernel<MODEL, G>(A.variant)<<<blocks, A.wpb * G, smem, st>>>(P, S, A);
   return cudaGetLastError();
 }
@@ -1472,12 +1395,15 @@ static cudaError_t launch_sweep_m(int G, const Problem& P, const DevState& S, co
   return cudaErrorInvalidValue;
 }
 
+// The shared memory a solve is accepted by: the chain and staged forms' layout.  The ring variant has always been
+// charged 2128 bytes more; windows in that margin fit the forms below without a ring.
+constexpr size_t kRingAllowance = 2128;
 size_t sweep_smem_bytes(const Problem& P, int wpb, int G, int variant) {
   size_t b = variant == kSweepStaged ? (size_t)wpb * ((size_t)P.w * 12 + (size_t)P.lat_words * 4)
                                      : (size_t)wpb * ((size_t)(P.w + 2 * kGuardBins) * 8 + (size_t)P.lat_words * 4);
   if (G > 1) b += (size_t)wpb * G * (variant == kSweepStaged ? sizeof(StagedTrial) : kChainStagingBytes);
   if (P.model == kEA || P.model == kEA3) b += (size_t)P.j_words * 4;
-  if (variant == kSweepRing) b += kRingBytes;
+  if (variant == kSweepRing) b += kRingAllowance;
   return b;
 }
 

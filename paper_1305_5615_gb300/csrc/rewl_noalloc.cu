@@ -24,10 +24,11 @@ namespace {
 
 // Working memory of one call, shared by all calls on a device:
 //   [0, 16)                       sweep clock (u64) and exchange round (u64)
+//   [16, 32)                      error word of the ring form's bounded waits (u32)
 //   then, each for REWL_NOALLOC_MAX_WALKERS walkers:
 //   active walker ids (i32), status flags (i32), accepted moves, near ties and
 //   exact tests (u64 each).
-constexpr size_t kClockBytes = 16;
+constexpr size_t kClockBytes = 32;
 constexpr size_t kMaxW = REWL_NOALLOC_MAX_WALKERS;
 constexpr size_t kScratchBytes = kClockBytes + kMaxW * (4 + 4 + 8 + 8 + 8);
 
@@ -138,6 +139,7 @@ extern "C" rewl_status rewl_sweep_noalloc(const rewl_sweep_desc* d, uint32_t* la
   S.win_start = const_cast<int32_t*>(win_start);
   S.lnf = const_cast<double*>(lnf);
   S.clock = reinterpret_cast<uint64_t*>(base);
+  S.error = reinterpret_cast<int32_t*>(base + 16);
   unsigned char* q = base + kClockBytes;
   S.active = reinterpret_cast<int32_t*>(q);
   q += kMaxW * 4;
@@ -170,6 +172,13 @@ extern "C" rewl_status rewl_sweep_noalloc(const rewl_sweep_desc* d, uint32_t* la
   A.n_active = (int)n_walkers;
   A.wpb = wpb;
   A.variant = kSweepChain;
+  A.wait_cycles = kDefaultWaitCycles;
+  // few walkers: each one's draws by warps of their own, as rewl_create chooses; only calls that end well within the
+  // bound of that form's waits (8 s; a trial of a walker takes 20 - 100 ns)
+  int dev = 0, n_sm = 0;
+  if (G == 32 && A.n_att <= (1u << 25) && cudaGetDevice(&dev) == cudaSuccess &&
+      cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n_walkers <= ring_walkers_per_sm(P) * n_sm)
+    A.variant = kSweepRing;
   if (launch_sweep(G, P, S, A, s) != cudaSuccess) {
     rewl_set_last_error("rewl_sweep_noalloc: sweep launch failed");
     return REWL_ECUDA;

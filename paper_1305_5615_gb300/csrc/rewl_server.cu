@@ -126,10 +126,10 @@ struct Group {
   BatchSlot* d_slots = nullptr;     // [cap]
   SlotReport* h_rep = nullptr;      // pinned [cap]
   SlotReport* d_rep = nullptr;      // [cap]
-  BatchWalker* h_list = nullptr;    // pinned [list_cap]: every walker, then (from n_list) every quad
+  BatchWalker* h_list = nullptr;    // pinned [list_cap]: every walker
   BatchWalker* d_list = nullptr;    // [list_cap]
-  int list_cap = 0, n_list = 0, n_quad = 0, hi = 0;  // hi: slots [0, hi) in the round
-  size_t smem = 0, smem_quad = 0;
+  int list_cap = 0, n_list = 0, hi = 0;  // hi: slots [0, hi) in the round
+  size_t smem[3] = {0, 0, 0};       // per BatchForm: the widest walker's
   int max_pairs = 0, max_m = 1, max_h = 1;
   bool dirty = true;
   // the captured replay: k rounds and the report, for one table and one sweep form
@@ -168,6 +168,7 @@ constexpr double kReplayMs = 4.0;  // target duration of one replay of a shared 
 constexpr double kPrivateReplayMs = 32.0;  // ... of a private group's (its request runs for seconds)
 constexpr double kPrivateRoundMs = 2.0;  // estimated round length from which requests get a group each
 constexpr int kMaxRoundsPerReplay = 16;
+constexpr int kRingWalkersPerSm = 5;  // of all groups together, up to which rounds run the ring form
 
 struct rewl_server {
   std::mutex mu;
@@ -325,28 +326,27 @@ struct rewl_server {
       g.d_rep = dr;
       g.cap = cap;
     }
-    int n = 0, nq = 0, hi = 0;
+    int n = 0, hi = 0;
     g.max_pairs = 0;
     g.max_m = 1;
     g.max_h = 1;
-    g.smem = 0;
-    g.smem_quad = 0;
+    for (size_t& b : g.smem) b = 0;
     for (int s = 0; s < need; ++s) {
       g.h_stage[s] = g.slots[s];
       if (!g.slot_req[s]) continue;
       const Problem& P = g.slots[s].P;
       n += P.n_walkers;
-      nq += (P.n_walkers + 3) / 4;
       hi = s + 1;
-      g.smem = std::max(g.smem, sweep_smem_bytes(P, 1, 32, kSweepChain));
-      g.smem_quad = std::max(g.smem_quad, sweep_smem_bytes(P, 4, 8, kSweepChain));
+      g.smem[kBatchOne] = std::max(g.smem[kBatchOne], resolve_smem(P, 1, false));
+      g.smem[kBatchRing] = std::max(g.smem[kBatchRing], resolve_smem(P, 1, true));
+      g.smem[kBatchChain] = std::max(g.smem[kBatchChain], sweep_smem_bytes(P, 1, 32, kSweepChain));
       g.max_pairs = std::max(g.max_pairs, P.h / 2);
       g.max_m = std::max(g.max_m, P.m);
       g.max_h = std::max(g.max_h, P.h);
     }
     g.hi = hi;
-    if (n + nq > g.list_cap) {
-      const int cap = std::max(n + nq, 2 * g.list_cap);
+    if (n > g.list_cap) {
+      const int cap = std::max(n, 2 * g.list_cap);
       BatchWalker *hl = nullptr, *dl = nullptr;
       if (cudaMallocHost(&hl, sizeof(BatchWalker) * cap) != cudaSuccess ||
           cudaMalloc(&dl, sizeof(BatchWalker) * cap) != cudaSuccess) {
@@ -365,15 +365,9 @@ struct rewl_server {
       if (!g.slot_req[s]) continue;
       for (int W = 0; W < g.slots[s].P.n_walkers; ++W) g.h_list[k++] = BatchWalker{s, W};
     }
-    for (int s = 0; s < hi; ++s) {
-      if (!g.slot_req[s]) continue;
-      for (int W = 0; W < g.slots[s].P.n_walkers; W += 4) g.h_list[k++] = BatchWalker{s, W};
-    }
     g.n_list = n;
-    g.n_quad = nq;
     if (hi) SCUDA(cudaMemcpyAsync(g.d_slots, g.h_stage, sizeof(BatchSlot) * hi, cudaMemcpyHostToDevice, g.stream));
-    if (n + nq)
-      SCUDA(cudaMemcpyAsync(g.d_list, g.h_list, sizeof(BatchWalker) * (n + nq), cudaMemcpyHostToDevice, g.stream));
+    if (n) SCUDA(cudaMemcpyAsync(g.d_list, g.h_list, sizeof(BatchWalker) * n, cudaMemcpyHostToDevice, g.stream));
     g.dirty = false;
     if (g.exec) {  // the replay read the old tables' sizes: capture again
       cudaGraphExecDestroy(g.exec);
@@ -389,14 +383,12 @@ struct rewl_server {
       cudaGraphExecDestroy(g.exec);
       g.exec = nullptr;
     }
-    const BatchWalker* list = form == kBatchQuad ? g.d_list + g.n_list : g.d_list;
-    const int n = form == kBatchQuad ? g.n_quad : g.n_list;
-    const size_t smem = form == kBatchQuad ? g.smem_quad : g.smem;
     cudaGraph_t graph = nullptr;
     SCUDA(cudaStreamBeginCapture(g.stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = cudaSuccess;
     for (int r = 0; r < g.k && e == cudaSuccess; ++r)
-      e = launch_round_batch(g.d_slots, g.hi, list, n, smem, g.max_pairs, g.max_m, g.max_h, form, g.model, g.stream);
+      e = launch_round_batch(g.d_slots, g.hi, g.d_list, g.n_list, g.smem[form], g.max_pairs, g.max_m, g.max_h, form, g.model,
+                             g.stream);
     if (e == cudaSuccess) e = launch_slot_report(g.d_slots, g.hi, g.d_rep, g.stream);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(g.h_rep, g.d_rep, sizeof(SlotReport) * g.hi, cudaMemcpyDeviceToHost, g.stream);
@@ -420,13 +412,12 @@ struct rewl_server {
       if (st != REWL_OK) return st;
     }
     if (g.n_list == 0) return REWL_OK;
-    // few walkers on the GPU: each walker's chain has a sub-partition to itself, and a producer
-    // warp per walker makes its draws (the ring form); many walkers share the SMs and their issue
-    // slots, and 4 walkers per CTA with 8 lanes each share the instructions of the sequential step
-    const bool few = active_walkers() <= 8 * n_sm;
-    int form = kBatchOne;
-    if (few && g.smem + ring_extra_smem() <= batch_smem_limit()) form = kBatchRing;
-    else if (!few && g.smem_quad <= batch_smem_limit()) form = kBatchQuad;
+    // few walkers on the GPU: each walker's passes are latency-bound, and producer warps make its
+    // draws (the ring form); many walkers share the SMs and their issue slots, and each makes its own
+    const bool few = active_walkers() <= kRingWalkersPerSm * n_sm;
+    int form = kBatchChain;
+    if (few && g.smem[kBatchRing] <= batch_smem_limit()) form = kBatchRing;
+    else if (g.smem[kBatchOne] <= batch_smem_limit()) form = kBatchOne;
     if (!g.exec || g.exec_form != form || g.exec_k != g.k) {
       rewl_status st = capture(g, form);
       if (st != REWL_OK) return st;
