@@ -203,11 +203,10 @@ struct OffsetBits {
     if constexpr (kNeighbours<MODEL> == 4 && MODEL != kPotts) {
       const uint32_t s0 = __ballot_sync(0xffffffffu, bonds & 1u), s1 = __ballot_sync(0xffffffffu, bonds & 2u),
                      s2 = __ballot_sync(0xffffffffu, bonds & 4u), s3 = __ballot_sync(0xffffffffu, bonds & 8u);
-      const uint32_t x = s0 ^ s1 ^ s2, y = (s0 & s1) | (s0 & s2) | (s1 & s2), z = x & s3;  // count = x + s3 + 2 y
-      const uint32_t c1 = y ^ z, c2 = y & z;
+      const uint32_t x = s0 ^ s1 ^ s2, y = (s0 & s1) | (s0 & s2) | (s1 & s2);  // count = x + s3 + 2 y
       b[0] = x ^ s3;  // count - 2 in two's complement
-      b[1] = ~c1;
-      b[2] = ~(c1 | c2);
+      b[1] = ~(y ^ (x & s3));
+      b[2] = ~(y | (x & s3));
     } else {
 #pragma unroll
       for (int k = 0; k < N; ++k) b[k] = __ballot_sync(0xffffffffu, (d >> k) & 1);
@@ -362,6 +361,7 @@ template <int MODEL>
 struct DrawRing {
   uint4 a[kRingGroups][32];  // site, right, left, down
   uint4 b[kRingGroups][32];  // up, aux, ln u (two words)
+  uint32_t touched[kRingGroups];  // trials at or next to whose site a later one of the group falls
   uint2 c[MODEL == kEA3 ? kRingGroups : 1][32];  // behind, in front
   uint32_t hits[kRingGroups][1 + kNeighbours<MODEL>][32];
   uint64_t full[kRingBatches], empty[kRingBatches];
@@ -404,6 +404,8 @@ __device__ __forceinline__ void produce_draws(const Problem& P, const DevState& 
       if ((h.s >> i1) & 1u) t1 |= kSelf;
       if ((h.s >> i2) & 1u) t2 |= kSelf;
       const bool many = __any_sync(0xffffffffu, (rest & (rest - 1u)) != 0u);
+      const uint32_t touched = __reduce_or_sync(0xffffffffu, around);
+      if (lane == 0) R.touched[sl] = touched;
       const uint32_t aux = (MODEL == kPotts ? d.pv : d.js) | i1 << 6 | i2 << 11 | t1 << 16 | t2 << 22 |
                            (many ? 1u << 31 : 0u);
       R.a[sl][lane] = make_uint4(row + d.x, row + d.xr, row + d.xl, (zo + d.yd) * L + d.x);
@@ -468,8 +470,7 @@ __device__ __forceinline__ void resolve_walker(const Problem& P, const DevState&
   // passes look at bits 24 .. 55 only (steps of 2^-16), the exact test follows where that is close.
   const int64_t clear = kGuardFx + ((int64_t)lane << lsh);
   const uint32_t clear_24 = (uint32_t)(clear >> 24) + 1u;
-  uint64_t n_acc = 0;
-  uint32_t n_tie = 0, n_exact = 0;
+  uint32_t n_acc = 0, n_tie = 0, n_exact = 0;  // of this lane's trials
   const uint32_t n_groups = (n_att + 31u) / 32u;
   const uint8_t* bytes = reinterpret_cast<const uint8_t*>(M.lat);
 
@@ -480,14 +481,18 @@ __device__ __forceinline__ void resolve_walker(const Problem& P, const DevState&
   // their decisions (A: the accepted ones) and what follows from them
   uint32_t A = 0u, v = 0u, nv = 0u;
   int d = 0, at = 0;
-  int post = -1;  // the bin the lane's trial of the previous group ended in (-1: none), not yet counted
+  int post = -1 - lane;  // the bin the lane's trial of the previous group ended in, not yet counted
+  uint32_t counting = 0u;  // the lanes that had a trial in it
   OffsetBits<MODEL> off;
 
   // The visits of a group: the last trial of every bin adds those of all (64-bit shared atomics are
-  // compare-and-swap loops: 143 cycles even alone); the others add nothing to an unused entry, without a branch.
+  // compare-and-swap loops: 143 cycles even alone); the others add to unused entries, without a branch.
   auto add_visits = [&](uint32_t same) {
-    const bool last = post >= 0 && (same >> lane) == 1u;
-    M.fx[last ? post : -1 - lane] += (int64_t)(last ? __popc(same) : 0) << lsh;
+    same &= counting;
+    const uint32_t n = __popc(same);
+    int64_t* f = &M.fx[(same >> lane) == 1u ? post : -1 - lane];
+    if constexpr (COUNT) *f += (int64_t)n << lsh;
+    else *f += (int64_t)((uint64_t)n * (1u << lsh));  // kexp >= kCountFrom: ln f is below 2^32 units
   };
   auto load_masks = [&](uint32_t g) {
     if constexpr (RING) {
@@ -511,9 +516,10 @@ __device__ __forceinline__ void resolve_walker(const Problem& P, const DevState&
 #pragma unroll
         for (int k = 0; k < 4; ++k) a[k] = last(A & h.n[k], n0[k]);
       } else {
-        const uint32_t i1 = (aux >> 6) & 31u, i2 = (aux >> 11) & 31u;
-        const uint32_t v1 = __shfl_sync(0xffffffffu, nv, i1), v2 = __shfl_sync(0xffffffffu, nv, i2);
-        const uint32_t t1 = (A >> i1) & 1u ? aux >> 16 : 0u, t2 = (A >> i2) & 1u ? aux >> 22 : 0u;  // i2 is the later
+        // shifts and shuffles take the low five bits of their counts
+        const uint32_t v1 = __shfl_sync(0xffffffffu, nv, aux >> 6), v2 = __shfl_sync(0xffffffffu, nv, aux >> 11);
+        const uint32_t t1 = __funnelshift_r(A, 0u, aux >> 6) & 1u ? aux >> 16 : 0u,
+                       t2 = __funnelshift_r(A, 0u, aux >> 11) & 1u ? aux >> 22 : 0u;  // the second is the later
         v = t2 & 16u ? v2 : t1 & 16u ? v1 : v0;
 #pragma unroll
         for (int k = 0; k < 4; ++k) a[k] = t2 & (1u << k) ? v2 : t1 & (1u << k) ? v1 : n0[k];
@@ -527,8 +533,8 @@ __device__ __forceinline__ void resolve_walker(const Problem& P, const DevState&
 #pragma unroll
         for (int k = 0; k < NB; ++k) bonds ^= (__popc(A & h.n[k]) & 1u) << k;
       } else {
-        const uint32_t on1 = 0u - ((A >> ((aux >> 6) & 31u)) & 1u), on2 = 0u - ((A >> ((aux >> 11) & 31u)) & 1u);
-        bonds ^= ((on1 & (aux >> 16)) ^ (on2 & (aux >> 22))) & kAll;
+        const uint32_t on1 = __funnelshift_r(A, 0u, aux >> 6) & 1u, on2 = __funnelshift_r(A, 0u, aux >> 11) & 1u;
+        bonds ^= on1 * ((aux >> 16) & kAll) ^ on2 * ((aux >> 22) & kAll);
       }
       d = offset_of_bonds<MODEL>(bonds);
       off.cut(d, bonds);
@@ -539,9 +545,8 @@ __device__ __forceinline__ void resolve_walker(const Problem& P, const DevState&
   int64_t gap = 0, f_old = 0, f_new = 0;  // gap: ln g(old) - ln g(new) - ln u
   int v_old = 0, v_new = 0;
   bool inwin = true;
-  auto pass = [&](auto masks, auto bin_bits, uint32_t& wide) -> uint32_t {
+  auto pass = [&](auto bin_bits, uint32_t& wide) -> uint32_t {
     constexpr int BITS = decltype(bin_bits)::value;
-    if (RING || touched) offset(masks);
     const int rel = off.sum(A & lt), to = rel + d;  // bins from the group's first
     at = bin + rel;
     inwin = (unsigned)(at + d) < (unsigned)w;
@@ -568,7 +573,8 @@ __device__ __forceinline__ void resolve_walker(const Problem& P, const DevState&
       uint32_t wide;
       do {
         const uint32_t was = nv;
-        const uint32_t B = (pass(std::true_type{}, std::integral_constant<int, 8>{}, wide) & ~fixed) | value;
+        offset(std::true_type{});
+        const uint32_t B = (pass(std::integral_constant<int, 8>{}, wide) & ~fixed) | value;
         again = B != A || (MODEL == kPotts && __any_sync(0xffffffffu, nv != was));
         A = B;
       } while (again);
@@ -596,9 +602,10 @@ __device__ __forceinline__ void resolve_walker(const Problem& P, const DevState&
   auto commit = [&](uint32_t g) {
     const bool acc = (A & bit) != 0u;
     atomicXor(&M.lat[site], (acc ? (MODEL == kPotts ? v ^ nv : 1u) : 0u) << shift);
-    post = thr > 0 ? -1 : acc ? at + d : at;
-    bin += off.sum(A);
-    n_acc += (uint64_t)__popc(A);
+    post = acc ? at + d : at;
+    counting = n_att - g * 32u >= 32u ? 0xffffffffu : (1u << (n_att - g * 32u)) - 1u;
+    bin = __shfl_sync(0xffffffffu, post, 31);
+    n_acc += acc;
     __syncwarp();
     if constexpr (RING) ring->release(g, lane);
   };
@@ -622,6 +629,7 @@ __device__ __forceinline__ void resolve_walker(const Problem& P, const DevState&
         shift = (a.x & 3u) * 8u;
         aux = b.y;
         thr = (int64_t)((uint64_t)b.z | (uint64_t)b.w << 32);
+        touched = ring->R.touched[g % kRingGroups];
         if constexpr (DENSE) load_masks(g);
         if (g + 1 < n_groups && !ring->fetch(g + 1, lane)) {
           stop = true;
@@ -681,12 +689,20 @@ __device__ __forceinline__ void resolve_walker(const Problem& P, const DevState&
         again = __any_sync(0xffffffffu, (A & bit) != 0u && (d != 0 || (touched & bit) != 0u));
       }
       while (again) {
-        const uint32_t was = nv;
-        uint32_t wide = 0u;
-        const uint32_t B = pass(Masks{}, std::integral_constant<int, COUNT ? kBinBits : 0>{}, wide);
-        leave = too_close() | wide;
-        again = B != A || (MODEL == kPotts && __any_sync(0xffffffffu, nv != was));
-        A = B;
+        // The offsets, for the accepted trials that touch others.  The passes that leave those alone need no new ones;
+        // where a group takes two passes, asking costs as much as that saves (the ring form at small ln f).
+        constexpr bool kEachPass = RING && !COUNT;
+        const uint32_t was = nv, by = A & touched;
+        if (RING || touched) offset(Masks{});
+        const bool moved = MODEL == kPotts && __any_sync(0xffffffffu, nv != was);  // proposed values others may build on
+        do {
+          uint32_t wide = 0u;
+          const uint32_t B = pass(std::integral_constant<int, COUNT ? kBinBits : 0>{}, wide);
+          leave = too_close() | wide;
+          again = B != A;
+          A = B;
+        } while (!kEachPass && again && (A & touched) == by);
+        again = again || moved;
       }
       if constexpr (!DENSE) leave |= aux >> 31;
       if (leave != 0u) break;
@@ -694,7 +710,7 @@ __device__ __forceinline__ void resolve_walker(const Problem& P, const DevState&
     }
     if (stop) {
       add_visits(__match_any_sync(0xffffffffu, post));
-      post = -1;
+      counting = 0u;
       break;
     }
     if (g < n_groups) {
@@ -709,6 +725,7 @@ __device__ __forceinline__ void resolve_walker(const Problem& P, const DevState&
   add_visits(__match_any_sync(0xffffffffu, post));
 
   for (int o = 16; o; o >>= 1) {
+    n_acc += __shfl_xor_sync(0xffffffffu, n_acc, o);
     n_tie += __shfl_xor_sync(0xffffffffu, n_tie, o);
     n_exact += __shfl_xor_sync(0xffffffffu, n_exact, o);
   }
