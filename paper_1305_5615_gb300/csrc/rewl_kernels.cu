@@ -1,7 +1,7 @@
 // rewl_kernels.cu -- the device phases of replica-exchange Wang-Landau:
 //   k_init_lattice  random start configurations and their energies
-//   k_descent       +-J: zero-temperature descent that fixes the energy range
-//   k_entry         greedy walk of every walker into its window
+//   k_greedy        +-J: zero-temperature descent that fixes the energy range;
+//                   greedy walk of every walker into its window
 //   k_sweep         the WL walk (paper, WL paragraph) -- the hot loop
 //   k_exchange      configuration swaps between neighbouring windows, Eq. (1)
 //   k_flat_merge    per-walker flatness, averaging of the window's ln g,
@@ -26,16 +26,6 @@ __device__ __forceinline__ uint32_t g_site(const Problem& P, const uint32_t* lat
   if (P.model == kPotts) return (lat[y * P.Wr + (x >> 3)] >> ((x & 7) * 4)) & 15u;
   return (lat[y * P.Wr + (x >> 5)] >> (x & 31)) & 1u;
 }
-__device__ __forceinline__ void g_set_site(const Problem& P, uint32_t* lat, int x, int y, uint32_t v) {
-  if (P.model == kPotts) {
-    uint32_t& wd = lat[y * P.Wr + (x >> 3)];
-    const int sh = (x & 7) * 4;
-    wd = (wd & ~(15u << sh)) | (v << sh);
-  } else {
-    uint32_t& wd = lat[y * P.Wr + (x >> 5)];
-    wd = (wd & ~(1u << (x & 31))) | (v << (x & 31));
-  }
-}
 // bond energy: Ising / +-J -J s_a s_b (bit 1 = spin -1, coupling bit 1 = J -1); Potts -delta
 __device__ __forceinline__ int bond_e(const Problem& P, uint32_t a, uint32_t b, uint32_t jneg) {
   if (P.model == kPotts) return a == b ? -1 : 0;
@@ -46,97 +36,58 @@ __device__ __forceinline__ uint32_t g_jbit(const Problem& P, const uint32_t* J, 
   if (P.model != kEA && P.model != kEA3) return 0u;
   return coupling_bit(J, P.Wr1, plane, P.rows, x, row);
 }
-__device__ int g_energy(const Problem& P, const uint32_t* lat, const uint32_t* J) {
+// ---------------------------------------------------------------------------
+// Start configurations: one warp a walker, a word of the configuration a lane.  Ising and +-J: site i is bit i % 32
+// of random word i / 32; Potts: site i is drawn from word i.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t init_word(const Problem& P, int W, uint32_t q) {
+  const U4 r = philox10(q >> 2, 0u, (uint32_t)W, kTagInit, P.seed_lo, P.seed_hi);
+  return (q & 3u) == 0 ? r.x : (q & 3u) == 1 ? r.y : (q & 3u) == 2 ? r.z : r.w;
+}
+
+// Energy of a configuration (global or shared memory) by a warp; the same for all lanes.
+__device__ int warp_energy(const Problem& P, const uint32_t* lat, const uint32_t* J) {
+  const int lane = threadIdx.x & 31, L = P.L;
   int E = 0;
-  const int L = P.L, nz = P.model == kEA3 ? L : 1;
-  for (int z = 0; z < nz; ++z)
-    for (int y = 0; y < L; ++y)
-      for (int x = 0; x < L; ++x) {
-        const int row = z * L + y;
-        const uint32_t s = g_site(P, lat, x, row);
-        const int xr = x + 1 == L ? 0 : x + 1, yd = y + 1 == L ? 0 : y + 1;
-        E += bond_e(P, s, g_site(P, lat, xr, row), g_jbit(P, J, 0, x, row));
-        E += bond_e(P, s, g_site(P, lat, x, z * L + yd), g_jbit(P, J, 1, x, row));
-        if (P.model == kEA3) {
-          const int zb = z + 1 == L ? 0 : z + 1;
-          E += bond_e(P, s, g_site(P, lat, x, zb * L + y), g_jbit(P, J, 2, x, row));
-        }
-      }
-  return E;
-}
-// energy change when site (x, y, z) takes value v (z = 0 in 2D)
-__device__ int g_delta_e(const Problem& P, const uint32_t* lat, const uint32_t* J, int x, int y, int z, uint32_t v) {
-  const int L = P.L;
-  const int xl = x ? x - 1 : L - 1, xr = x + 1 == L ? 0 : x + 1;
-  const int yu = y ? y - 1 : L - 1, yd = y + 1 == L ? 0 : y + 1;
-  const int zo = z * L, row = zo + y;
-  const uint32_t s = g_site(P, lat, x, row);
-  const uint32_t nr = g_site(P, lat, xr, row), nl = g_site(P, lat, xl, row);
-  const uint32_t nd = g_site(P, lat, x, zo + yd), nu = g_site(P, lat, x, zo + yu);
-  const uint32_t jr = g_jbit(P, J, 0, x, row), jl = g_jbit(P, J, 0, xl, row);
-  const uint32_t jd = g_jbit(P, J, 1, x, row), ju = g_jbit(P, J, 1, x, zo + yu);
-  int before = bond_e(P, s, nr, jr) + bond_e(P, s, nl, jl) + bond_e(P, s, nd, jd) + bond_e(P, s, nu, ju);
-  int after = bond_e(P, v, nr, jr) + bond_e(P, v, nl, jl) + bond_e(P, v, nd, jd) + bond_e(P, v, nu, ju);
-  if (P.model == kEA3) {
-    const int zf = z ? z - 1 : L - 1, zb = z + 1 == L ? 0 : z + 1;
-    const uint32_t nb = g_site(P, lat, x, zb * L + y), nf = g_site(P, lat, x, zf * L + y);
-    const uint32_t jb = g_jbit(P, J, 2, x, row), jf = g_jbit(P, J, 2, x, zf * L + y);
-    before += bond_e(P, s, nb, jb) + bond_e(P, s, nf, jf);
-    after += bond_e(P, v, nb, jb) + bond_e(P, v, nf, jf);
-  }
-  return after - before;
-}
-
-// The site of a draw: (x, y) on the square lattice, (x, y, z) on the cube.
-__device__ __forceinline__ void decode_site(const Problem& P, uint32_t site, int& x, int& y, int& z) {
-  if (P.model == kEA3) {
-    z = (int)mulhi32(site, P.magic_L2);
-    site -= (uint32_t)z * (uint32_t)(P.L * P.L);
-  } else {
-    z = 0;
-  }
-  y = (int)mulhi32(site, P.magic_L);
-  x = (int)site - y * P.L;
-}
-
-__device__ __forceinline__ void propose(const Problem& P, const uint32_t* lat, const U4& r, int& x, int& y, int& z,
-                                        uint32_t& v) {
-  const uint32_t site = scale32(r.x, (uint32_t)P.N);
-  decode_site(P, site, x, y, z);
-  const uint32_t s = g_site(P, lat, x, z * P.L + y);
-  if (P.model == kPotts) {
-    v = s + 1u + scale32(r.y, (uint32_t)(P.q - 1));
-    if (v >= (uint32_t)P.q) v -= (uint32_t)P.q;
-  } else {
-    v = s ^ 1u;
-  }
-}
-
-// ---------------------------------------------------------------------------
-// Set-up kernels (one thread per walker)
-// ---------------------------------------------------------------------------
-__global__ void k_init_lattice(Problem P, DevState S) {
-  const int W = blockIdx.x * blockDim.x + threadIdx.x;
-  if (W >= P.n_walkers) return;
-  uint32_t* lat = S.lat + (size_t)W * P.lat_words;
-  for (int i = 0; i < P.lat_words; ++i) lat[i] = 0u;
-  U4 r{0, 0, 0, 0};
-  for (int i = 0; i < P.N; ++i) {
-    const int x = i % P.L, y = i / P.L;
-    if (P.model == kPotts) {
-      if ((i & 3) == 0) r = philox10((uint32_t)(i >> 2), 0u, (uint32_t)W, kTagInit, P.seed_lo, P.seed_hi);
-      const uint32_t w = (i & 3) == 0 ? r.x : (i & 3) == 1 ? r.y : (i & 3) == 2 ? r.z : r.w;
-      g_set_site(P, lat, x, y, scale32(w, (uint32_t)P.q));
-    } else {
-      if ((i & 127) == 0) r = philox10((uint32_t)(i >> 7), 0u, (uint32_t)W, kTagInit, P.seed_lo, P.seed_hi);
-      const int wi = (i & 127) >> 5;
-      const uint32_t w = wi == 0 ? r.x : wi == 1 ? r.y : wi == 2 ? r.z : r.w;
-      g_set_site(P, lat, x, y, (w >> (i & 31)) & 1u);
+  for (int i = lane; i < P.N; i += 32) {
+    const int row = i / L, x = i - row * L, z = row / L, y = row - z * L;  // z = 0 in 2D
+    const uint32_t s = g_site(P, lat, x, row);
+    const int xr = x + 1 == L ? 0 : x + 1, yd = y + 1 == L ? 0 : y + 1;
+    E += bond_e(P, s, g_site(P, lat, xr, row), g_jbit(P, J, 0, x, row));
+    E += bond_e(P, s, g_site(P, lat, x, z * L + yd), g_jbit(P, J, 1, x, row));
+    if (P.model == kEA3) {
+      const int zb = z + 1 == L ? 0 : z + 1;
+      E += bond_e(P, s, g_site(P, lat, x, zb * L + y), g_jbit(P, J, 2, x, row));
     }
   }
-  S.E[W] = g_energy(P, lat, S.J);
-  S.entry_t[W] = 0;
-  S.status[W] = 0;
+  for (int o = 16; o; o >>= 1) E += __shfl_xor_sync(0xffffffffu, E, o);
+  return E;
+}
+
+__global__ void __launch_bounds__(128) k_init_lattice(Problem P, DevState S) {
+  const int W = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (W >= P.n_walkers) return;
+  uint32_t* lat = S.lat + (size_t)W * P.lat_words;
+  const int per = P.model == kPotts ? 8 : 32;
+  for (int i = lane; i < P.lat_words; i += 32) {
+    const int row = i / P.Wr, x0 = (i - row * P.Wr) * per, n = min(per, P.L - x0);
+    const uint32_t site = (uint32_t)(row * P.L + x0);
+    uint32_t word = 0u;
+    if (P.model == kPotts) {
+      for (int k = 0; k < n; ++k) word |= scale32(init_word(P, W, site + k), (uint32_t)P.q) << (4 * k);
+    } else {
+      word = __funnelshift_r(init_word(P, W, site >> 5), init_word(P, W, (site >> 5) + 1u), site & 31u);
+      if (n < 32) word &= (1u << n) - 1u;
+    }
+    lat[i] = word;
+  }
+  __syncwarp();
+  const int E = warp_energy(P, lat, S.J);
+  if (lane == 0) {
+    S.E[W] = E;
+    S.entry_t[W] = 0;
+    S.status[W] = 0;
+  }
 }
 
 __device__ __forceinline__ int window_distance(int E, int lo, int hi) { return E < lo ? lo - E : (E > hi ? E - hi : 0); }
@@ -146,46 +97,6 @@ __device__ __forceinline__ int window_distance(int E, int lo, int hi) { return E
 // always the largest width and the stride of the per-walker ln g and H rows.
 __device__ __forceinline__ int window_width(const Problem& P, const DevState& S, int a) {
   return S.win_width ? S.win_width[a] : P.w;
-}
-
-// One greedy move on the entry stream.  target < 0: minimise E (descent);
-// otherwise minimise the distance to window `target`.
-__device__ void greedy_move(const Problem& P, DevState& S, uint32_t* lat, int W, int lo, int hi, bool descent) {
-  const uint64_t t = S.entry_t[W]++;
-  const U4 r = philox10((uint32_t)t, (uint32_t)(t >> 32), (uint32_t)W, kTagEntry, P.seed_lo, P.seed_hi);
-  int x, y, z;
-  uint32_t v;
-  propose(P, lat, r, x, y, z, v);
-  const int E = S.E[W];
-  const int En = E + g_delta_e(P, lat, S.J, x, y, z, v);
-  const int before = descent ? E : window_distance(E, lo, hi);
-  const int after = descent ? En : window_distance(En, lo, hi);
-  if (after <= before) {
-    g_set_site(P, lat, x, z * P.L + y, v);
-    S.E[W] = En;
-  }
-}
-
-__global__ void k_descent(Problem P, DevState S, uint64_t n_att) {
-  const int W = blockIdx.x * blockDim.x + threadIdx.x;
-  if (W >= P.n_walkers) return;
-  uint32_t* lat = S.lat + (size_t)W * P.lat_words;
-  for (uint64_t n = 0; n < n_att; ++n) greedy_move(P, S, lat, W, 0, 0, true);
-}
-
-__global__ void k_entry(Problem P, DevState S, uint64_t budget) {
-  const int W = blockIdx.x * blockDim.x + threadIdx.x;
-  if (W >= P.n_walkers) return;
-  uint32_t* lat = S.lat + (size_t)W * P.lat_words;
-  const int a = W / P.m;
-  const int lo = P.e_min + S.win_start[a] * P.e_step;
-  const int hi = P.e_min + (S.win_start[a] + window_width(P, S, a) - 1) * P.e_step;
-  for (uint64_t n = 0; n < budget && window_distance(S.E[W], lo, hi) > 0; ++n) greedy_move(P, S, lat, W, lo, hi, false);
-  if (window_distance(S.E[W], lo, hi) == 0) return;
-  for (int i = 0; i < P.lat_words; ++i) lat[i] = S.seed_config[i];
-  S.E[W] = g_energy(P, lat, S.J);
-  for (uint64_t n = 0; n < budget && window_distance(S.E[W], lo, hi) > 0; ++n) greedy_move(P, S, lat, W, lo, hi, false);
-  if (window_distance(S.E[W], lo, hi) != 0) S.status[W] = 5;  // REWL_EENTRY
 }
 
 // ---------------------------------------------------------------------------
@@ -913,6 +824,122 @@ __device__ __forceinline__ void sweep_chain_body(const Problem& P, const DevStat
 #include "rewl_resolve.cuh"
 namespace rewl {
 
+// ---------------------------------------------------------------------------
+// Set-up walks on a walker's entry stream, 32 moves decided together as in the sweeps (one warp a walker):
+// descent -- moves that do not raise the energy; entry -- moves that do not lead further from the window, until the
+// walker is in it.  One thread a walker, on its configuration in global memory, was bound by the latency of one move
+// after the other (about 0.5 us).  rewl_create before -> after: Potts q = 10 32 x 32, 512 walkers 348 -> 16 ms; +-J
+// 32 x 32 78 -> 3.0 ms, 12^3 158 -> 5.7 ms; Ising 128 x 128, 4096 walkers 900 -> 35 ms; Ising 32 x 32 1.7 -> 0.41 ms.
+// ---------------------------------------------------------------------------
+template <int MODEL>
+__device__ __forceinline__ void greedy_walk(const Problem& P, const DevState& S, uint32_t* lat, uint32_t* tab, int W,
+                                            uint64_t& t, int& E, int lo, int hi, bool descent, uint64_t budget) {
+  constexpr int NB = kNeighbours<MODEL>;
+  const int lane = threadIdx.x & 31;
+  const uint32_t bit = 1u << lane, lt = bit - 1u;
+  const uint64_t end = t + budget;
+  while (t < end && (descent || window_distance(E, lo, hi) > 0)) {
+    const uint64_t i = t + (uint64_t)lane;
+    const U4 r = philox10((uint32_t)i, (uint32_t)(i >> 32), (uint32_t)W, kTagEntry, P.seed_lo, P.seed_hi);
+    const TrialDraw dr = place_trial<MODEL>(P, S.J, r);
+    const TrialHits<MODEL> h = find_hits<MODEL>(tab, P.L, dr, lane);
+    const TrialBase<MODEL> b = base_of<MODEL>(P, lat, dr);
+    uint32_t A = 0u, v = b.v, nv = 0u;
+    int d = 0, before = E;
+    if constexpr (MODEL == kPotts) potts_move((uint32_t)P.q, dr.pv, v, b.n[0], b.n[1], b.n[2], b.n[3], nv);
+    OffsetBits<MODEL> off;
+    bool again = true;
+    while (again) {
+      const uint32_t was = nv;
+      uint32_t bonds = b.sat;
+      if constexpr (MODEL == kPotts) {
+        auto last = [&](uint32_t m, uint32_t old) {
+          const uint32_t got = __shfl_sync(0xffffffffu, nv, m ? 31 - __clz(m) : lane);
+          return m ? got : old;
+        };
+        v = last(A & h.s, b.v);
+        const uint32_t n0 = last(A & h.n[0], b.n[0]), n1 = last(A & h.n[1], b.n[1]), n2 = last(A & h.n[2], b.n[2]),
+                       n3 = last(A & h.n[3], b.n[3]);
+        d = potts_move((uint32_t)P.q, dr.pv, v, n0, n1, n2, n3, nv);
+      } else {
+        bonds ^= (__popc(A & h.s) & 1) ? (1u << NB) - 1u : 0u;
+#pragma unroll
+        for (int k = 0; k < NB; ++k) bonds ^= (__popc(A & h.n[k]) & 1u) << k;
+        d = offset_of_bonds<MODEL>(bonds);
+      }
+      off.cut(d, bonds);
+      before = E + P.e_step * off.sum(A & lt);
+      const int after = before + P.e_step * d;
+      const bool acc = i < end && (descent ? d <= 0 : window_distance(after, lo, hi) <= window_distance(before, lo, hi));
+      const uint32_t B = __ballot_sync(0xffffffffu, acc);
+      again = B != A || (MODEL == kPotts && __any_sync(0xffffffffu, nv != was));
+      A = B;
+    }
+    int n = (int)(end - t < 32ull ? end - t : 32ull);
+    if (!descent) {  // the walk ends with the first move after which the walker is in its window
+      const int now = before + ((A & bit) ? P.e_step * d : 0);
+      const uint32_t in = __ballot_sync(0xffffffffu, lane < n && window_distance(now, lo, hi) == 0);
+      if (in) n = __ffs(in);
+    }
+    A &= n >= 32 ? 0xffffffffu : (1u << n) - 1u;
+    if (A & bit) atomicXor(&lat[b.widx], (MODEL == kPotts ? v ^ nv : 1u) << b.shift);
+    E += P.e_step * off.sum(A);
+    t += (uint64_t)n;
+    __syncwarp();
+  }
+}
+
+// One warp a CTA and walker.  descent: n moves; else into the window, again from the seed configuration if the first
+// walk does not get there in n moves.
+template <int MODEL>
+__global__ void __launch_bounds__(32) k_greedy(Problem P, DevState S, bool descent, uint64_t n) {
+  extern __shared__ uint32_t s_greedy[];
+  uint32_t *tab = s_greedy, *lat = s_greedy + kHitTables<MODEL> * P.L;
+  const int W = blockIdx.x, lane = threadIdx.x;
+  uint32_t* g_lat = S.lat + (size_t)W * P.lat_words;
+  for (int i = lane; i < kHitTables<MODEL> * P.L; i += 32) tab[i] = 0u;
+  for (int i = lane; i < P.lat_words; i += 32) lat[i] = g_lat[i];
+  __syncwarp();
+  uint64_t t = S.entry_t[W];
+  int E = S.E[W];
+  if (descent) {
+    greedy_walk<MODEL>(P, S, lat, tab, W, t, E, 0, 0, true, n);
+  } else {
+    const int a = W / P.m;
+    const int lo = P.e_min + S.win_start[a] * P.e_step;
+    const int hi = P.e_min + (S.win_start[a] + window_width(P, S, a) - 1) * P.e_step;
+    greedy_walk<MODEL>(P, S, lat, tab, W, t, E, lo, hi, false, n);
+    if (window_distance(E, lo, hi) > 0) {
+      for (int i = lane; i < P.lat_words; i += 32) lat[i] = S.seed_config[i];
+      __syncwarp();
+      E = warp_energy(P, lat, S.J);
+      greedy_walk<MODEL>(P, S, lat, tab, W, t, E, lo, hi, false, n);
+      if (window_distance(E, lo, hi) != 0 && lane == 0) S.status[W] = 5;  // REWL_EENTRY
+    }
+  }
+  for (int i = lane; i < P.lat_words; i += 32) g_lat[i] = lat[i];
+  if (lane == 0) {
+    S.E[W] = E;
+    S.entry_t[W] = t;
+  }
+}
+
+template <int MODEL>
+static cudaError_t launch_greedy_m(const Problem& P, const DevState& S, bool descent, uint64_t n, cudaStream_t st) {
+  const size_t smem = ((size_t)kHitTables<MODEL> * P.L + P.lat_words) * sizeof(uint32_t);  // at most 34 KB
+  k_greedy<MODEL><<<P.n_walkers, 32, smem, st>>>(P, S, descent, n);
+  return cudaGetLastError();
+}
+static cudaError_t launch_greedy(const Problem& P, const DevState& S, bool descent, uint64_t n, cudaStream_t st) {
+  switch (P.model) {
+    case kIsing: return launch_greedy_m<kIsing>(P, S, descent, n, st);
+    case kPotts: return launch_greedy_m<kPotts>(P, S, descent, n, st);
+    case kEA: return launch_greedy_m<kEA>(P, S, descent, n, st);
+    case kEA3: return launch_greedy_m<kEA3>(P, S, descent, n, st);
+  }
+  return cudaErrorInvalidValue;
+}
+
 // wpb walkers a CTA, one warp each, every group of 32 trials decided together.  Bound by issue (72% of the
 // active cycles, the integer pipe 69%): 24 warps an SM at 80 registers; 64 registers for 32 warps spill and lose 6%.
 constexpr int kResolveWarps = 2;  // most walkers a CTA: they share nothing but the couplings
@@ -1444,18 +1471,16 @@ cudaError_t launch_flat_merge(const Problem& P, const DevState& S, cudaStream_t 
 }
 
 cudaError_t launch_init(const Problem& P, const DevState& S, cudaStream_t st) {
-  k_init_lattice<<<(P.n_walkers + 63) / 64, 64, 0, st>>>(P, S);
+  k_init_lattice<<<(P.n_walkers + 3) / 4, 128, 0, st>>>(P, S);
   return cudaGetLastError();
 }
 
 cudaError_t launch_descent(const Problem& P, const DevState& S, uint64_t n_att, cudaStream_t st) {
-  k_descent<<<(P.n_walkers + 63) / 64, 64, 0, st>>>(P, S, n_att);
-  return cudaGetLastError();
+  return launch_greedy(P, S, true, n_att, st);
 }
 
 cudaError_t launch_entry(const Problem& P, const DevState& S, uint64_t budget, cudaStream_t st) {
-  k_entry<<<(P.n_walkers + 63) / 64, 64, 0, st>>>(P, S, budget);
-  return cudaGetLastError();
+  return launch_greedy(P, S, false, budget, st);
 }
 
 }  // namespace rewl

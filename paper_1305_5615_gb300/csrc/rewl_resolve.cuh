@@ -70,15 +70,14 @@ struct TrialHits {
   }
 };
 
+// Site, neighbours and proposal of the draw r (all of a TrialDraw but thr).
 template <int MODEL>
-__device__ __forceinline__ TrialDraw draw_trial(const Problem& P, const uint32_t* s_J, uint64_t t, int W) {
-  const U4 r = philox10((uint32_t)t, (uint32_t)(t >> 32), (uint32_t)W, kTagFlip, P.seed_lo, P.seed_hi);
+__device__ __forceinline__ TrialDraw place_trial(const Problem& P, const uint32_t* J, const U4& r) {
   int x, y;
   uint32_t pv;
   trial_site<MODEL>(P, r, x, y, pv);
-  const float uf = __ull2float_rn(2ull * u52_bits(r.z, r.w) + 1ull) * 0x1p-53f;
   TrialDraw d;
-  d.thr = __float2ll_rn(logf(uf) * 1099511627776.0f);
+  d.thr = 0;
   const uint32_t L = (uint32_t)P.L;
   d.x = (uint32_t)x;
   d.y = (uint32_t)y;
@@ -89,18 +88,27 @@ __device__ __forceinline__ TrialDraw draw_trial(const Problem& P, const uint32_t
   d.z = d.zb = d.zf = d.pv = d.js = 0u;
   if constexpr (MODEL == kPotts) d.pv = pv;
   if constexpr (MODEL == kEA) {
-    d.js = coupling_bit(s_J, P.Wr1, 0, L, d.x, d.y) | coupling_bit(s_J, P.Wr1, 0, L, d.xl, d.y) << 1 |
-           coupling_bit(s_J, P.Wr1, 1, L, d.x, d.y) << 2 | coupling_bit(s_J, P.Wr1, 1, L, d.x, d.yu) << 3;
+    d.js = coupling_bit(J, P.Wr1, 0, L, d.x, d.y) | coupling_bit(J, P.Wr1, 0, L, d.xl, d.y) << 1 |
+           coupling_bit(J, P.Wr1, 1, L, d.x, d.y) << 2 | coupling_bit(J, P.Wr1, 1, L, d.x, d.yu) << 3;
   }
   if constexpr (MODEL == kEA3) {
     d.z = pv;
     d.zb = pv + 1u == L ? 0u : pv + 1u;
     d.zf = (pv ? pv : L) - 1u;
     const uint32_t zo = pv * L, R = (uint32_t)P.rows;
-    d.js = coupling_bit(s_J, P.Wr1, 0, R, d.x, zo + d.y) | coupling_bit(s_J, P.Wr1, 0, R, d.xl, zo + d.y) << 1 |
-           coupling_bit(s_J, P.Wr1, 1, R, d.x, zo + d.y) << 2 | coupling_bit(s_J, P.Wr1, 1, R, d.x, zo + d.yu) << 3 |
-           coupling_bit(s_J, P.Wr1, 2, R, d.x, zo + d.y) << 4 | coupling_bit(s_J, P.Wr1, 2, R, d.x, d.zf * L + d.y) << 5;
+    d.js = coupling_bit(J, P.Wr1, 0, R, d.x, zo + d.y) | coupling_bit(J, P.Wr1, 0, R, d.xl, zo + d.y) << 1 |
+           coupling_bit(J, P.Wr1, 1, R, d.x, zo + d.y) << 2 | coupling_bit(J, P.Wr1, 1, R, d.x, zo + d.yu) << 3 |
+           coupling_bit(J, P.Wr1, 2, R, d.x, zo + d.y) << 4 | coupling_bit(J, P.Wr1, 2, R, d.x, d.zf * L + d.y) << 5;
   }
+  return d;
+}
+
+template <int MODEL>
+__device__ __forceinline__ TrialDraw draw_trial(const Problem& P, const uint32_t* J, uint64_t t, int W) {
+  const U4 r = philox10((uint32_t)t, (uint32_t)(t >> 32), (uint32_t)W, kTagFlip, P.seed_lo, P.seed_hi);
+  TrialDraw d = place_trial<MODEL>(P, J, r);
+  const float uf = __ull2float_rn(2ull * u52_bits(r.z, r.w) + 1ull) * 0x1p-53f;
+  d.thr = __float2ll_rn(logf(uf) * 1099511627776.0f);
   return d;
 }
 
