@@ -19,58 +19,139 @@
 
 namespace {
 
-__device__ __forceinline__ double block_reduce(double v, double* sh, bool is_max) {
+// Sum over the CTA, the same for all threads.  The warps' sums are added up by the first warp alone: done by every
+// thread, these few additions were half of the FP64 pipe's work.
+__device__ __forceinline__ double block_sum(double v, double* sh) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-  for (int o = 16; o; o >>= 1) {
-    const double u = __shfl_xor_sync(0xffffffffu, v, o);
-    v = is_max ? fmax(v, u) : v + u;
-  }
-  __syncthreads();
+  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (nw == 1) return v;
+  __syncthreads();  // the last sum has been read
   if (lane == 0) sh[wid] = v;
   __syncthreads();
-  double r = sh[0];
-  for (int i = 1; i < nw; ++i) r = is_max ? fmax(r, sh[i]) : r + sh[i];
-  return r;
+  if (wid == 0) {
+    double r = lane < nw ? sh[lane] : 0.0;
+    for (int o = 4; o; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);  // at most eight warps
+    __syncwarp();
+    if (lane == 0) sh[0] = r;
+  }
+  __syncthreads();
+  return sh[0];
+}
+__device__ __forceinline__ long long block_max(long long v, long long* sh) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+  for (int o = 16; o; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+  if (lane == 0) sh[wid] = v;
+  __syncthreads();
+  for (int i = 0; i < nw; ++i) v = max(v, sh[i]);
+  return v;
+}
+
+// 2^(j/64), rounded.
+__device__ const double kExp2[64] = {
+    0x1.0000000000000p+0, 0x1.02c9a3e778061p+0, 0x1.059b0d3158574p+0, 0x1.0874518759bc8p+0,
+    0x1.0b5586cf9890fp+0, 0x1.0e3ec32d3d1a2p+0, 0x1.11301d0125b51p+0, 0x1.1429aaea92de0p+0,
+    0x1.172b83c7d517bp+0, 0x1.1a35beb6fcb75p+0, 0x1.1d4873168b9aap+0, 0x1.2063b88628cd6p+0,
+    0x1.2387a6e756238p+0, 0x1.26b4565e27cddp+0, 0x1.29e9df51fdee1p+0, 0x1.2d285a6e4030bp+0,
+    0x1.306fe0a31b715p+0, 0x1.33c08b26416ffp+0, 0x1.371a7373aa9cbp+0, 0x1.3a7db34e59ff7p+0,
+    0x1.3dea64c123422p+0, 0x1.4160a21f72e2ap+0, 0x1.44e086061892dp+0, 0x1.486a2b5c13cd0p+0,
+    0x1.4bfdad5362a27p+0, 0x1.4f9b2769d2ca7p+0, 0x1.5342b569d4f82p+0, 0x1.56f4736b527dap+0,
+    0x1.5ab07dd485429p+0, 0x1.5e76f15ad2148p+0, 0x1.6247eb03a5585p+0, 0x1.6623882552225p+0,
+    0x1.6a09e667f3bcdp+0, 0x1.6dfb23c651a2fp+0, 0x1.71f75e8ec5f74p+0, 0x1.75feb564267c9p+0,
+    0x1.7a11473eb0187p+0, 0x1.7e2f336cf4e62p+0, 0x1.82589994cce13p+0, 0x1.868d99b4492edp+0,
+    0x1.8ace5422aa0dbp+0, 0x1.8f1ae99157736p+0, 0x1.93737b0cdc5e5p+0, 0x1.97d829fde4e50p+0,
+    0x1.9c49182a3f090p+0, 0x1.a0c667b5de565p+0, 0x1.a5503b23e255dp+0, 0x1.a9e6b5579fdbfp+0,
+    0x1.ae89f995ad3adp+0, 0x1.b33a2b84f15fbp+0, 0x1.b7f76f2fb5e47p+0, 0x1.bcc1e904bc1d2p+0,
+    0x1.c199bdd85529cp+0, 0x1.c67f12e57d14bp+0, 0x1.cb720dcef9069p+0, 0x1.d072d4a07897cp+0,
+    0x1.d5818dcfba487p+0, 0x1.da9e603db3285p+0, 0x1.dfc97337b9b5fp+0, 0x1.e502ee78b3ff6p+0,
+    0x1.ea4afa2a490dap+0, 0x1.efa1bee615a27p+0, 0x1.f50765b6e4540p+0, 0x1.fa7c1819e90d8p+0,
+};
+
+// exp(x) for -746 < x <= 0 by a table of 2^(j/64) and a polynomial on the rest (P. T. P. Tang, Table-driven
+// implementation of the exponential function, ACM TOMS 15, 144 (1989)): x = n ln2/64 + r, |r| <= ln2/128, and
+// e^r - 1 to r^5 (the next term is below 3.5e-17).  Ten FP64 operations: the FP64 pipe (2.2 lane operations a
+// cycle and SM) is what bounds these sums.  tab: kExp2 in shared memory.
+__device__ __forceinline__ double exp_of_nonpositive(double x, const double* tab) {
+  constexpr double kMagic = 6755399441055744.0;  // 1.5 * 2^52: the sum's low word is the rounded integer
+  const double t = fma(x, 0x1.71547652b82fep+6, kMagic);
+  const int n = __double2loint(t);
+  const double f = t - kMagic;
+  const double r = fma(f, -0x1.abc9e3b39803fp-62, fma(f, -0x1.62e42fefa39efp-7, x));
+  double q = fma(r, 1.0 / 120.0, 1.0 / 24.0);
+  q = fma(r, q, 1.0 / 6.0);
+  q = fma(r, q, 0.5);
+  const double s = tab[n & 63];
+  const double v = fma(s, fma(r * r, q, r), s);
+  const int k = n >> 6;  // -1077 .. 0
+  if (k >= -1021) return __hiloint2double(__double2hiint(v) + (k << 20), __double2loint(v));
+  return __hiloint2double(__double2hiint(v) + ((k + 128) << 20), __double2loint(v)) * 0x1p-128;  // into the denormals
 }
 
 // One CTA per (temperature, table): table blockIdx.y of n_bins values, output
-// [table][temperature][5].
-__global__ void k_thermo(const double* __restrict__ lng_tables, int n_bins, int e_min, int e_step,
-                         const double* __restrict__ T, double* __restrict__ out_tables) {
-  __shared__ double sh[32];
+// [table][temperature][5].  Each weight is computed once and kept in shared memory for the
+// centred moment (s_w holds n_bins of them, or none and they are computed again); a term of
+// exp(-746) or less, which is 0 in FP64, is not computed at all; the largest term is found
+// on the integer pipe.  rewl_thermo_jackknife of 8 runs of 1025 levels at 300 temperatures
+// (2700 CTAs) before -> after: 583 -> 348 us a call, with CUDA's exp 451.
+constexpr uint32_t kZeroHi = 0x40875000u;  // upper word of 746
+__device__ __forceinline__ long long order_key(double v) {  // orders as the numbers do (no NaN)
+  const long long i = __double_as_longlong(v);
+  return i ^ (long long)((unsigned long long)(i >> 63) >> 1);
+}
+__global__ void __launch_bounds__(256) k_thermo(const double* __restrict__ lng_tables, int n_bins, int e_min,
+                                                int e_step, const double* __restrict__ T,
+                                                double* __restrict__ out_tables, int keep) {
+  extern __shared__ double s_w[];
+  __shared__ double sh[8], tab[64];
+  __shared__ long long sh_max[8];
   const double* lng = lng_tables + (size_t)blockIdx.y * n_bins;
   double* out = out_tables + (size_t)blockIdx.y * gridDim.x * 5;
   const double t = T[blockIdx.x];
   const double beta = 1.0 / t;
-  double mx = -INFINITY;
-  for (int b = threadIdx.x; b < n_bins; b += blockDim.x) {
+  for (int j = threadIdx.x; j < 64; j += blockDim.x) tab[j] = kExp2[j];  // block_max synchronises before its use
+  // E of the thread's bins: integers well below 2^53, so the steps are exact
+  const double e_first = (double)(e_min + (int)threadIdx.x * e_step), e_stride = (double)blockDim.x * (double)e_step;
+  long long top = order_key(-INFINITY);
+  double e = e_first;
+  for (int b = threadIdx.x; b < n_bins; b += blockDim.x, e += e_stride) {
     const double l = lng[b];
-    if (isfinite(l)) mx = fmax(mx, l - beta * (double)(e_min + b * e_step));
+    const double a = isfinite(l) ? l - beta * e : -INFINITY;
+    if (keep) s_w[b] = a;  // its own thread reads it back
+    top = max(top, order_key(a));
   }
-  mx = block_reduce(mx, sh, true);
+  top = block_max(top, sh_max);
+  const double mx = __longlong_as_double(top ^ (long long)((unsigned long long)(top >> 63) >> 1));
   double z = 0.0, ze = 0.0;
-  for (int b = threadIdx.x; b < n_bins; b += blockDim.x) {
-    const double l = lng[b];
-    if (isfinite(l)) {
-      const double E = (double)(e_min + b * e_step);
-      const double wgt = exp(l - beta * E - mx);
+  e = e_first;
+  for (int b = threadIdx.x; b < n_bins; b += blockDim.x, e += e_stride) {
+    const double a = keep ? s_w[b] : isfinite(lng[b]) ? lng[b] - beta * e : -INFINITY;
+    const double x = a - mx;
+    double wgt = 0.0;
+    if ((uint32_t)(__double2hiint(x) & 0x7fffffff) < kZeroHi) {  // |x| < 746
+      wgt = exp_of_nonpositive(x, tab);
       z += wgt;
-      ze += wgt * E;
+      ze += wgt * e;
     }
+    if (keep) s_w[b] = wgt;
   }
-  z = block_reduce(z, sh, false);
-  ze = block_reduce(ze, sh, false);
+  z = block_sum(z, sh);
+  ze = block_sum(ze, sh);
   const double U = ze / z;
   double zc = 0.0;
-  for (int b = threadIdx.x; b < n_bins; b += blockDim.x) {
-    const double l = lng[b];
-    if (isfinite(l)) {
-      const double E = (double)(e_min + b * e_step);
-      const double d = E - U;
-      zc += exp(l - beta * E - mx) * d * d;
+  e = e_first;
+  for (int b = threadIdx.x; b < n_bins; b += blockDim.x, e += e_stride) {
+    double wgt = 0.0;
+    if (keep) {
+      wgt = s_w[b];
+    } else {
+      const double x = (isfinite(lng[b]) ? lng[b] - beta * e : -INFINITY) - mx;
+      if ((uint32_t)(__double2hiint(x) & 0x7fffffff) < kZeroHi) wgt = exp_of_nonpositive(x, tab);
+    }
+    if (__double_as_longlong(wgt) != 0) {
+      const double d = e - U;
+      zc += wgt * d * d;
     }
   }
-  zc = block_reduce(zc, sh, false);
+  zc = block_sum(zc, sh);
   if (threadIdx.x == 0) {
     const double lnZ = mx + log(z);
     const double F = -t * lnZ;
@@ -81,6 +162,18 @@ __global__ void k_thermo(const double* __restrict__ lng_tables, int n_bins, int 
     o[3] = F;
     o[4] = (U - F) / t;
   }
+}
+
+constexpr int kKeepBins = 4096;  // weights kept up to here: 32 KB of shared memory, seven CTAs an SM
+// Threads a CTA: few temperatures and tables are latency-bound, eight warps each; many fill the SMs, and then fewer
+// warps share out a table, with fewer additions across warps (that call with 256 threads 388 us, 128 353, 64 348).
+constexpr int kFewCtas = 304;  // two an SM
+void launch_thermo(const double* tables, int n_tables, int n_bins, int e_min, int e_step, const double* T, int n_T,
+                   double* out) {
+  const int keep = n_bins <= kKeepBins;
+  const int threads = (int64_t)n_T * n_tables <= kFewCtas || n_bins > 8192 ? 256 : n_bins > 2048 ? 128 : 64;
+  k_thermo<<<dim3(n_T, (unsigned)n_tables), threads, keep ? sizeof(double) * n_bins : 0>>>(tables, n_bins, e_min, e_step,
+                                                                                          T, out, keep);
 }
 
 // Jackknife tables: [0] the mean ln g over the R runs, [1 + i] the mean
@@ -171,7 +264,7 @@ extern "C" rewl_status rewl_thermo_jackknife(const double* lng_runs, int32_t n_r
   }
   if (st == REWL_OK) {
     k_jack_tables<<<(n_bins + 255) / 256, 256>>>(d_runs, n_runs, n_bins, d_tab);
-    k_thermo<<<dim3(n_T, (unsigned)nt), 256>>>(d_tab, n_bins, e_min, e_step, d_T, d_q);
+    launch_thermo(d_tab, (int)nt, n_bins, e_min, e_step, d_T, n_T, d_q);
     k_jack_combine<<<(n_T * 5 + 127) / 128, 128>>>(d_q, n_runs, n_T, d_est, d_err);
     if (cudaGetLastError() != cudaSuccess ||
         cudaMemcpy(est, d_est, sizeof(double) * n_T * 5, cudaMemcpyDeviceToHost) != cudaSuccess ||
@@ -215,7 +308,7 @@ extern "C" rewl_status rewl_thermo(const double* lng, int32_t n_bins, int32_t e_
     st = REWL_ECUDA;
   }
   if (st == REWL_OK) {
-    k_thermo<<<dim3(n_T, 1), 256>>>(d_lng, n_bins, e_min, e_step, d_T, d_out);
+    launch_thermo(d_lng, 1, n_bins, e_min, e_step, d_T, n_T, d_out);
     if (cudaGetLastError() != cudaSuccess ||
         cudaMemcpy(out, d_out, sizeof(double) * 5 * n_T, cudaMemcpyDeviceToHost) != cudaSuccess) {
       rewl_set_last_error("rewl_thermo: kernel failed");
