@@ -12,7 +12,7 @@
 
 #include <cmath>
 #include <cstdint>
-#include <vector>
+#include <mutex>
 
 #include "rewl.h"
 #include "rewl_ctx.h"
@@ -214,6 +214,47 @@ __global__ void k_jack_combine(const double* __restrict__ q, int R, int n_T, dou
   err[j] = sqrt(__dmul_rn(__ddiv_rn((double)(R - 1), (double)R), ss));
 }
 
+// A call's device memory, one block: a fixed array of the library while it fits (32 runs of 1025 levels at 300
+// temperatures do), held by one call at a time, else an allocation.  Allocating and releasing the only block of a
+// process maps and unmaps a page of device memory: 59 us of the 107 us that the smallest call took.  The array's
+// address is looked up in every call and belongs to the current device.
+constexpr size_t kScratchDoubles = 1u << 17;
+static __device__ double g_thermo_scratch[kScratchDoubles];
+std::mutex g_scratch_mutex;
+struct DeviceBlock {
+  double* d = nullptr;
+  bool own = false;
+  std::unique_lock<std::mutex> lock;
+  explicit DeviceBlock(size_t n) {
+    if (n <= kScratchDoubles) {
+      lock = std::unique_lock<std::mutex>(g_scratch_mutex);
+      void* p = nullptr;
+      if (cudaGetSymbolAddress(&p, g_thermo_scratch) == cudaSuccess) {
+        d = static_cast<double*>(p);
+        return;
+      }
+      lock.unlock();
+    }
+    own = cudaMalloc(&d, sizeof(double) * n) == cudaSuccess;
+    if (!own) d = nullptr;
+  }
+  ~DeviceBlock() {
+    if (own) cudaFree(d);
+  }
+  DeviceBlock(const DeviceBlock&) = delete;
+  DeviceBlock& operator=(const DeviceBlock&) = delete;
+};
+bool to_device(double* d, const double* h, size_t n) {
+  return cudaMemcpy(d, h, sizeof(double) * n, cudaMemcpyHostToDevice) == cudaSuccess;
+}
+bool from_device(double* h, const double* d, size_t n) {
+  return cudaMemcpy(h, d, sizeof(double) * n, cudaMemcpyDeviceToHost) == cudaSuccess;
+}
+rewl_status failed(rewl_status st, const char* msg) {
+  rewl_set_last_error(msg);
+  return st;
+}
+
 rewl_status check_temperatures(const double* temperatures, int32_t n_T) {
   for (int i = 0; i < n_T; ++i)
     if (!(temperatures[i] > 0.0) || !std::isfinite(temperatures[i])) {
@@ -244,42 +285,19 @@ extern "C" rewl_status rewl_thermo_jackknife(const double* lng_runs, int32_t n_r
     rewl_set_last_error("rewl_thermo_jackknife: no bin is finite in every run");
     return REWL_EINVAL;
   }
-  const size_t nt = (size_t)n_runs + 1;
-  double *d_runs = nullptr, *d_tab = nullptr, *d_T = nullptr, *d_q = nullptr, *d_est = nullptr, *d_err = nullptr;
-  rewl_status st = REWL_OK;
-  if (cudaMalloc(&d_runs, sizeof(double) * n_runs * (size_t)n_bins) != cudaSuccess ||
-      cudaMalloc(&d_tab, sizeof(double) * nt * n_bins) != cudaSuccess ||
-      cudaMalloc(&d_T, sizeof(double) * n_T) != cudaSuccess ||
-      cudaMalloc(&d_q, sizeof(double) * nt * n_T * 5) != cudaSuccess ||
-      cudaMalloc(&d_est, sizeof(double) * n_T * 5) != cudaSuccess ||
-      cudaMalloc(&d_err, sizeof(double) * n_T * 5) != cudaSuccess) {
-    rewl_set_last_error("rewl_thermo_jackknife: device allocation failed");
-    st = REWL_ENOMEM;
-  }
-  if (st == REWL_OK &&
-      (cudaMemcpy(d_runs, lng_runs, sizeof(double) * n_runs * (size_t)n_bins, cudaMemcpyHostToDevice) != cudaSuccess ||
-       cudaMemcpy(d_T, temperatures, sizeof(double) * n_T, cudaMemcpyHostToDevice) != cudaSuccess)) {
-    rewl_set_last_error("rewl_thermo_jackknife: copy failed");
-    st = REWL_ECUDA;
-  }
-  if (st == REWL_OK) {
-    k_jack_tables<<<(n_bins + 255) / 256, 256>>>(d_runs, n_runs, n_bins, d_tab);
-    launch_thermo(d_tab, (int)nt, n_bins, e_min, e_step, d_T, n_T, d_q);
-    k_jack_combine<<<(n_T * 5 + 127) / 128, 128>>>(d_q, n_runs, n_T, d_est, d_err);
-    if (cudaGetLastError() != cudaSuccess ||
-        cudaMemcpy(est, d_est, sizeof(double) * n_T * 5, cudaMemcpyDeviceToHost) != cudaSuccess ||
-        cudaMemcpy(err, d_err, sizeof(double) * n_T * 5, cudaMemcpyDeviceToHost) != cudaSuccess) {
-      rewl_set_last_error("rewl_thermo_jackknife: kernel failed");
-      st = REWL_ECUDA;
-    }
-  }
-  cudaFree(d_runs);
-  cudaFree(d_tab);
-  cudaFree(d_T);
-  cudaFree(d_q);
-  cudaFree(d_est);
-  cudaFree(d_err);
-  return st;
+  const size_t nt = (size_t)n_runs + 1, n_in = (size_t)n_runs * n_bins, n_out = (size_t)n_T * 5;
+  DeviceBlock mem((size_t)n_T + n_in + nt * n_bins + nt * n_out + 2 * n_out);
+  if (!mem.d) return failed(REWL_ENOMEM, "rewl_thermo_jackknife: device allocation failed");
+  double *d_T = mem.d, *d_runs = d_T + n_T, *d_tab = d_runs + n_in, *d_q = d_tab + nt * n_bins;
+  double *d_est = d_q + nt * n_out, *d_err = d_est + n_out;
+  if (!to_device(d_T, temperatures, n_T) || !to_device(d_runs, lng_runs, n_in))
+    return failed(REWL_ECUDA, "rewl_thermo_jackknife: copy failed");
+  k_jack_tables<<<(n_bins + 255) / 256, 256>>>(d_runs, n_runs, n_bins, d_tab);
+  launch_thermo(d_tab, (int)nt, n_bins, e_min, e_step, d_T, n_T, d_q);
+  k_jack_combine<<<(n_T * 5 + 127) / 128, 128>>>(d_q, n_runs, n_T, d_est, d_err);
+  if (cudaGetLastError() != cudaSuccess || !from_device(est, d_est, n_out) || !from_device(err, d_err, n_out))
+    return failed(REWL_ECUDA, "rewl_thermo_jackknife: kernel failed");
+  return REWL_OK;
 }
 
 extern "C" rewl_status rewl_thermo(const double* lng, int32_t n_bins, int32_t e_min, int32_t e_step,
@@ -295,28 +313,13 @@ extern "C" rewl_status rewl_thermo(const double* lng, int32_t n_bins, int32_t e_
     rewl_set_last_error("rewl_thermo: no finite ln g");
     return REWL_EINVAL;
   }
-  double *d_lng = nullptr, *d_T = nullptr, *d_out = nullptr;
-  rewl_status st = REWL_OK;
-  if (cudaMalloc(&d_lng, sizeof(double) * n_bins) != cudaSuccess || cudaMalloc(&d_T, sizeof(double) * n_T) != cudaSuccess ||
-      cudaMalloc(&d_out, sizeof(double) * 5 * n_T) != cudaSuccess) {
-    rewl_set_last_error("rewl_thermo: device allocation failed");
-    st = REWL_ENOMEM;
-  }
-  if (st == REWL_OK && (cudaMemcpy(d_lng, lng, sizeof(double) * n_bins, cudaMemcpyHostToDevice) != cudaSuccess ||
-                        cudaMemcpy(d_T, temperatures, sizeof(double) * n_T, cudaMemcpyHostToDevice) != cudaSuccess)) {
-    rewl_set_last_error("rewl_thermo: copy failed");
-    st = REWL_ECUDA;
-  }
-  if (st == REWL_OK) {
-    launch_thermo(d_lng, 1, n_bins, e_min, e_step, d_T, n_T, d_out);
-    if (cudaGetLastError() != cudaSuccess ||
-        cudaMemcpy(out, d_out, sizeof(double) * 5 * n_T, cudaMemcpyDeviceToHost) != cudaSuccess) {
-      rewl_set_last_error("rewl_thermo: kernel failed");
-      st = REWL_ECUDA;
-    }
-  }
-  cudaFree(d_lng);
-  cudaFree(d_T);
-  cudaFree(d_out);
-  return st;
+  DeviceBlock mem((size_t)n_T + n_bins + 5 * (size_t)n_T);
+  if (!mem.d) return failed(REWL_ENOMEM, "rewl_thermo: device allocation failed");
+  double *d_T = mem.d, *d_lng = d_T + n_T, *d_out = d_lng + n_bins;
+  if (!to_device(d_T, temperatures, n_T) || !to_device(d_lng, lng, n_bins))
+    return failed(REWL_ECUDA, "rewl_thermo: copy failed");
+  launch_thermo(d_lng, 1, n_bins, e_min, e_step, d_T, n_T, d_out);
+  if (cudaGetLastError() != cudaSuccess || !from_device(out, d_out, 5 * (size_t)n_T))
+    return failed(REWL_ECUDA, "rewl_thermo: kernel failed");
+  return REWL_OK;
 }
