@@ -392,7 +392,7 @@ rewl_status rewl_create(rewl_handle* out, const rewl_model* model, const rewl_la
   S.status = (int32_t*)c->dalloc(sizeof(int32_t) * nW, &st);
   S.entry_t = (uint64_t*)c->dalloc(sizeof(uint64_t) * nW, &st);
   S.seed_config = (uint32_t*)c->dalloc(sizeof(uint32_t) * P.lat_words, &st);
-  S.clock = (uint64_t*)c->dalloc(sizeof(uint64_t) * 3, &st);
+  S.clock = (uint64_t*)c->dalloc(sizeof(uint64_t) * 4, &st);
   if (st != REWL_OK) return bail(st);
   cudaStream_t s = c->stream;
 #define BAIL_CUDA(expr)                                                                                   \
@@ -422,7 +422,7 @@ rewl_status rewl_create(rewl_handle* out, const rewl_model* model, const rewl_la
   BAIL_CUDA(cudaMemsetAsync(S.x_tried, 0, sizeof(uint64_t) * P.h, s));
   BAIL_CUDA(cudaMemsetAsync(S.x_accepted, 0, sizeof(uint64_t) * P.h, s));
   BAIL_CUDA(cudaMemsetAsync(S.seed_config, 0, sizeof(uint32_t) * P.lat_words, s));
-  BAIL_CUDA(cudaMemsetAsync(S.clock, 0, sizeof(uint64_t) * 3, s));
+  BAIL_CUDA(cudaMemsetAsync(S.clock, 0, sizeof(uint64_t) * 4, s));
   BAIL_CUDA(launch_init(P, S, s));
 
   // energy range
@@ -577,8 +577,7 @@ static rewl_status enqueue_block(rewl_ctx* c, bool with_flat) {
     c->pre_t0[k2] = t0n;
     c->pre_cur = k2;
   }
-  CUDA_TRY(launch_exchange(c->P, c->S, c->stream));
-  CUDA_TRY(launch_advance_clock(c->S, (uint32_t)c->params.sweeps_per_exchange, c->stream));
+  CUDA_TRY(launch_exchange(c->P, c->S, (uint32_t)c->params.sweeps_per_exchange, c->stream));
   if (with_flat) CUDA_TRY(launch_flat_merge(c->P, c->S, c->stream));
   return REWL_OK;
 }

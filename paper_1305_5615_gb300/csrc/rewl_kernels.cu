@@ -1022,25 +1022,30 @@ cudaError_t launch_precompute(int G, const Problem& P, uint64_t t0, uint32_t n_a
 // ---------------------------------------------------------------------------
 // Replica exchange, Eq. (1).  One CTA per window pair (a, a+1), a = round
 // (mod 2); walker k of window a is paired with walker sigma(k) of window a+1,
-// sigma a Fisher-Yates permutation from the round's own stream.
+// sigma a Fisher-Yates permutation from the round's own stream: its draws by
+// all threads, its swaps by one.  A pair is decided by one thread, its
+// configurations are exchanged by a warp (a thread alone, word after word, took
+// most of the kernel: 9 - 18 us at 32 words a walker).
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void exchange_body(const Problem& P, const DevState& S, int pair_block) {
-  extern __shared__ int sigma[];
-  const uint32_t round = (uint32_t)S.clock[1];
+__device__ __forceinline__ void exchange_body(const Problem& P, const DevState& S, int pair_block, uint32_t round) {
+  extern __shared__ int sigma[];  // [m], then [m] draws and flags
   const int a = 2 * pair_block + (int)(round & 1u);
   if (a + 1 >= P.h) return;
   if (S.done[a] || S.done[a + 1]) return;
   const int m = P.m;
-  if (threadIdx.x == 0) {
-    for (int k = 0; k < m; ++k) sigma[k] = k;
+  int* flag = sigma + m;
+  for (int i = threadIdx.x; i < m; i += blockDim.x) {
+    sigma[i] = i;
+    const U4 r = philox10(round, (uint32_t)a, (uint32_t)i, kTagPerm, P.seed_lo, P.seed_hi);
+    flag[i] = (int)scale32(r.x, (uint32_t)(i + 1));
+  }
+  __syncthreads();
+  if (threadIdx.x == 0)
     for (int i = m - 1; i >= 1; --i) {
-      const U4 r = philox10(round, (uint32_t)a, (uint32_t)i, kTagPerm, P.seed_lo, P.seed_hi);
-      const int j = (int)scale32(r.x, (uint32_t)(i + 1));
-      const int tmp = sigma[i];
+      const int j = flag[i], tmp = sigma[i];
       sigma[i] = sigma[j];
       sigma[j] = tmp;
     }
-  }
   __syncthreads();
   const int loA = P.e_min + S.win_start[a] * P.e_step, hiA = loA + (window_width(P, S, a) - 1) * P.e_step;
   const int loB = P.e_min + S.win_start[a + 1] * P.e_step, hiB = loB + (window_width(P, S, a + 1) - 1) * P.e_step;
@@ -1048,30 +1053,26 @@ __device__ __forceinline__ void exchange_body(const Problem& P, const DevState& 
   for (int k = threadIdx.x; k < m; k += blockDim.x) {
     const int Wi = a * m + k, Wj = (a + 1) * m + sigma[k];
     const int EX = S.E[Wi], EY = S.E[Wj];
-    if (EX < loB || EX > hiB || EY < loA || EY > hiA) continue;
-    const double* gi = S.lng + (size_t)Wi * P.w;
-    const double* gj = S.lng + (size_t)Wj * P.w;
-    const int iX = (EX - loA) / P.e_step, iY = (EY - loA) / P.e_step;
-    const int jX = (EX - loB) / P.e_step, jY = (EY - loB) / P.e_step;
-    const double d1 = __dsub_rn(gi[iX], gi[iY]);
-    const double d2 = __dsub_rn(gj[jY], gj[jX]);
-    const double D = __dadd_rn(d1, d2);
-    bool acc = D >= 0.0;
-    if (!acc) {
-      const U4 r = philox10(round, (uint32_t)a, (uint32_t)k, kTagXacc, P.seed_lo, P.seed_hi);
-      const double u = __dmul_rn(__ull2double_rn(2ull * u52_bits(r.z, r.w) + 1ull), 0x1p-53);
-      const double lu = log(u);
-      if (fabs(__dsub_rn(lu, D)) < 1e-12) S.near_ties[Wi] += 1;
-      acc = lu < D;
-    }
-    if (acc) {
-      uint32_t* li = S.lat + (size_t)Wi * P.lat_words;
-      uint32_t* lj = S.lat + (size_t)Wj * P.lat_words;
-      for (int i = 0; i < P.lat_words; ++i) {
-        const uint32_t t = li[i];
-        li[i] = lj[i];
-        lj[i] = t;
+    bool acc = false;
+    if (EX >= loB && EX <= hiB && EY >= loA && EY <= hiA) {
+      const double* gi = S.lng + (size_t)Wi * P.w;
+      const double* gj = S.lng + (size_t)Wj * P.w;
+      const int iX = (EX - loA) / P.e_step, iY = (EY - loA) / P.e_step;
+      const int jX = (EX - loB) / P.e_step, jY = (EY - loB) / P.e_step;
+      const double d1 = __dsub_rn(gi[iX], gi[iY]);
+      const double d2 = __dsub_rn(gj[jY], gj[jX]);
+      const double D = __dadd_rn(d1, d2);
+      acc = D >= 0.0;
+      if (!acc) {
+        const U4 r = philox10(round, (uint32_t)a, (uint32_t)k, kTagXacc, P.seed_lo, P.seed_hi);
+        const double u = __dmul_rn(__ull2double_rn(2ull * u52_bits(r.z, r.w) + 1ull), 0x1p-53);
+        const double lu = log(u);
+        if (fabs(__dsub_rn(lu, D)) < 1e-12) S.near_ties[Wi] += 1;
+        acc = lu < D;
       }
+    }
+    flag[k] = acc;
+    if (acc) {
       S.E[Wi] = EY;
       S.E[Wj] = EX;
       ++n_acc;
@@ -1087,11 +1088,45 @@ __device__ __forceinline__ void exchange_body(const Problem& P, const DevState& 
       }
     }
   }
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  for (int k = threadIdx.x >> 5; k < m; k += blockDim.x >> 5) {
+    if (!flag[k]) continue;
+    uint32_t* li = S.lat + (size_t)(a * m + k) * P.lat_words;
+    uint32_t* lj = S.lat + (size_t)((a + 1) * m + sigma[k]) * P.lat_words;
+    for (int i = lane; i < P.lat_words; i += 32) {
+      const uint32_t t = li[i];
+      li[i] = lj[i];
+      lj[i] = t;
+    }
+  }
   if (n_acc) atomicAdd(reinterpret_cast<unsigned long long*>(&S.x_accepted[a]), (unsigned long long)n_acc);
   if (threadIdx.x == 0) atomicAdd(reinterpret_cast<unsigned long long*>(&S.x_tried[a]), (unsigned long long)m);
 }
 
-__global__ void k_exchange(Problem P, DevState S) { exchange_body(P, S, (int)blockIdx.x); }
+constexpr int kExchangeThreads = 128;
+
+// Whether a CTA of the exchange is the last of `ctas` to be done with the round: that one moves the clocks on, which
+// was a launch of its own (2.5 us).  clock[3] counts the CTAs.
+__device__ __forceinline__ bool last_of(uint64_t* clock, int ctas) {
+  __shared__ bool last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(reinterpret_cast<unsigned long long*>(&clock[3]), 1ull) == (unsigned long long)(ctas - 1);
+    if (last) clock[3] = 0;
+  }
+  __syncthreads();
+  return last;
+}
+
+__global__ void k_exchange(Problem P, DevState S, uint32_t sweeps) {
+  exchange_body(P, S, (int)blockIdx.x, (uint32_t)S.clock[1]);
+  if (last_of(S.clock, gridDim.x) && threadIdx.x == 0) {
+    S.clock[0] += sweeps;
+    S.clock[1] += 1;
+  }
+}
 
 // ---------------------------------------------------------------------------
 // Flatness, merge and f update.  One CTA per window.
@@ -1225,23 +1260,28 @@ __global__ void __launch_bounds__(RING ? kRingThreads : 32, RING ? kRingCtas : 1
   else sweep_resolve_body<MODEL>(P, S, n_att, &bw.W, 1);
 }
 
+// Clocks of a slot after a round: the sweeps, the round, the trials of the walkers that ran.
+__device__ __forceinline__ void advance_slot(const BatchSlot& slot) {
+  const int h = slot.P.h, nd = *slot.S.n_done;  // windows done before this round's check
+  if (nd >= h) return;                          // finished: the clocks stay
+  uint64_t* clk = slot.S.clock;
+  clk[0] += slot.spe;
+  clk[1] += 1;
+  clk[2] += (uint64_t)(h - nd) * (uint64_t)slot.P.m * slot.n_att;
+}
+
 __global__ void k_exchange_batch(const BatchSlot* __restrict__ slots, int max_pairs) {
   const int s = (int)blockIdx.x / max_pairs, p = (int)blockIdx.x % max_pairs;
   if (!slots[s].active) return;
   const Problem P = slots[s].P;
   const DevState S = slots[s].S;
-  exchange_body(P, S, p);
+  exchange_body(P, S, p, (uint32_t)S.clock[1]);
+  if (last_of(S.clock, max_pairs) && threadIdx.x == 0) advance_slot(slots[s]);
 }
 
 __global__ void k_advance_batch(const BatchSlot* __restrict__ slots, int n_slots) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= n_slots || !slots[s].active) return;
-  const int h = slots[s].P.h, nd = *slots[s].S.n_done;  // windows done before this round's check
-  if (nd >= h) return;                                   // finished: the clocks stay
-  uint64_t* clk = slots[s].S.clock;
-  clk[0] += slots[s].spe;
-  clk[1] += 1;
-  clk[2] += (uint64_t)(h - nd) * (uint64_t)slots[s].P.m * slots[s].n_att;
+  if (s < n_slots && slots[s].active) advance_slot(slots[s]);
 }
 
 __global__ void k_flat_batch(const BatchSlot* __restrict__ slots, int max_h) {
@@ -1311,10 +1351,10 @@ cudaError_t launch_round_batch(const BatchSlot* d_slots, int n_slots, const Batc
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (max_pairs > 0) {
-    const int threads = max_m < 128 ? ((max_m + 31) / 32) * 32 : 128;
-    k_exchange_batch<<<n_slots * max_pairs, threads, (size_t)max_m * sizeof(int), st>>>(d_slots, max_pairs);
+    k_exchange_batch<<<n_slots * max_pairs, kExchangeThreads, 2 * (size_t)max_m * sizeof(int), st>>>(d_slots, max_pairs);
+  } else {  // single windows only
+    k_advance_batch<<<(n_slots + 127) / 128, 128, 0, st>>>(d_slots, n_slots);
   }
-  k_advance_batch<<<(n_slots + 127) / 128, 128, 0, st>>>(d_slots, n_slots);
   k_flat_batch<<<n_slots * max_h, 256, 0, st>>>(d_slots, max_h);
   return cudaGetLastError();
 }
@@ -1446,22 +1486,16 @@ cudaError_t launch_sweep(int G, const Problem& P, const DevState& S, const Sweep
   return cudaErrorInvalidValue;
 }
 
-// One CTA per possible pair of either parity; CTAs of the other parity exit.
-cudaError_t launch_exchange(const Problem& P, const DevState& S, cudaStream_t st) {
-  const int pairs = P.h / 2;
-  if (pairs <= 0) return cudaSuccess;
-  const int threads = P.m < 128 ? ((P.m + 31) / 32) * 32 : 128;
-  k_exchange<<<pairs, threads, (size_t)P.m * sizeof(int), st>>>(P, S);
-  return cudaGetLastError();
-}
-
 __global__ void k_advance_clock(DevState S, uint32_t sweeps) {
   S.clock[0] += sweeps;
   S.clock[1] += 1;
 }
 
-cudaError_t launch_advance_clock(const DevState& S, uint32_t sweeps, cudaStream_t st) {
-  k_advance_clock<<<1, 1, 0, st>>>(S, sweeps);
+// The exchange round and the clocks after it.  One CTA per possible pair of either parity.
+cudaError_t launch_exchange(const Problem& P, const DevState& S, uint32_t sweeps, cudaStream_t st) {
+  const int pairs = P.h / 2;
+  if (pairs > 0) k_exchange<<<pairs, kExchangeThreads, 2 * (size_t)P.m * sizeof(int), st>>>(P, S, sweeps);
+  else k_advance_clock<<<1, 1, 0, st>>>(S, sweeps);
   return cudaGetLastError();
 }
 

@@ -54,7 +54,8 @@ struct DevState {
   int32_t* status;       // per walker: 0 ok, else a rewl_status
   uint64_t* entry_t;     // per walker counter of the entry stream
   uint32_t* seed_config; // restart configuration for the entry walk
-  uint64_t* clock;       // [0] sweeps done by the solve, [1] exchange rounds done, [2] trials (batched rounds)
+  uint64_t* clock;       // [0] sweeps done by the solve, [1] exchange rounds done, [2] trials (batched rounds),
+                         // [3] CTAs of the exchange that are done with the round
   int32_t* stage;        // [h] 1/t rule: 0 = halving on the histogram test, 1 = following 1/t
   int32_t* win_width;    // [h] bins of each window (NULL: P.w for all)
   int64_t* first_iter;   // [h] sweep clock of each window's first merge, -1 before (may be NULL)
