@@ -1248,14 +1248,21 @@ __global__ void __launch_bounds__(32, 16) k_sweep_batch(const BatchSlot* __restr
 
 // The forms that decide 32 trials together, one walker per CTA: with producer warps for rounds with few walkers on
 // the GPU (each walker's passes are latency-bound), without for rounds with many (the issue slots are what runs out).
+// Registers for 5 and 24 walkers an SM, without spills; with the slot's sizes and pointers in registers and 7 ring CTAs
+// an SM (80 registers, 72 bytes spilled) a served batch of 24 requests took 512 ms, now 450.
 template <int MODEL, bool RING>
-__global__ void __launch_bounds__(RING ? kRingThreads : 32, RING ? kRingCtas : 16) k_sweep_batch_resolve(
+__global__ void __launch_bounds__(RING ? kRingThreads : 32, RING ? kBatchRingCtas : 24) k_sweep_batch_resolve(
     const BatchSlot* __restrict__ slots, const BatchWalker* __restrict__ list) {
+  // the slot in shared memory: as locals its sizes and pointers would take the registers that the passes need
+  __shared__ __align__(16) BatchSlot slot;
   const BatchWalker bw = list[blockIdx.x];
-  const Problem P = slots[bw.slot].P;
-  const DevState S = slots[bw.slot].S;
-  const uint32_t n_att = slots[bw.slot].n_att;
-  if (!slots[bw.slot].active || S.done[bw.W / P.m]) return;  // uniform over the CTA
+  const uint32_t* src = reinterpret_cast<const uint32_t*>(&slots[bw.slot]);
+  for (int i = threadIdx.x; i < (int)(sizeof(BatchSlot) / 4); i += blockDim.x) reinterpret_cast<uint32_t*>(&slot)[i] = src[i];
+  __syncthreads();
+  const Problem& P = slot.P;
+  const DevState& S = slot.S;
+  const uint32_t n_att = slot.n_att;
+  if (!slot.active || S.done[bw.W / P.m]) return;  // uniform over the CTA
   if constexpr (RING) sweep_resolve_ring_body<MODEL>(P, S, n_att, bw.W, kDefaultWaitCycles);
   else sweep_resolve_body<MODEL>(P, S, n_att, &bw.W, 1);
 }

@@ -31,6 +31,7 @@ cudaError_t launch_round_batch(const BatchSlot* d_slots, int n_slots, const Batc
                                cudaStream_t st);
 // forms of the batched sweep, one walker per CTA: 32 trials decided together, the same with
 // producer warps, and the chain form (windows too wide for the others' tables)
+constexpr int kBatchRingCtas = 5;  // ring CTAs (walkers) an SM holds; rounds with more active walkers run kBatchOne
 enum BatchForm : int { kBatchOne = 0, kBatchRing = 1, kBatchChain = 2 };
 cudaError_t launch_slot_report(const BatchSlot* d_slots, int n_slots, SlotReport* out, cudaStream_t st);
 

@@ -168,7 +168,6 @@ constexpr double kReplayMs = 4.0;  // target duration of one replay of a shared 
 constexpr double kPrivateReplayMs = 32.0;  // ... of a private group's (its request runs for seconds)
 constexpr double kPrivateRoundMs = 2.0;  // estimated round length from which requests get a group each
 constexpr int kMaxRoundsPerReplay = 16;
-constexpr int kRingWalkersPerSm = 5;  // of all groups together, up to which rounds run the ring form
 
 struct rewl_server {
   std::mutex mu;
@@ -414,7 +413,7 @@ struct rewl_server {
     if (g.n_list == 0) return REWL_OK;
     // few walkers on the GPU: each walker's passes are latency-bound, and producer warps make its
     // draws (the ring form); many walkers share the SMs and their issue slots, and each makes its own
-    const bool few = active_walkers() <= kRingWalkersPerSm * n_sm;
+    const bool few = active_walkers() <= kBatchRingCtas * n_sm;
     int form = kBatchChain;
     if (few && g.smem[kBatchRing] <= batch_smem_limit()) form = kBatchRing;
     else if (g.smem[kBatchOne] <= batch_smem_limit()) form = kBatchOne;
