@@ -96,7 +96,7 @@ typedef struct {
   int32_t profile;               /* 1 = time every sweep launch with CUDA events on the solve's stream
                                     (plain mode); read back through rewl_info */
   int32_t sweep_variant;         /* sweep kernel form, identical results: REWL_SWEEP_AUTO (default: the
-                                    ring form when its CTAs, one a walker, run in one wave (7 per SM; fewer for
+                                    ring form when its CTAs, one a walker, run in one wave (6 per SM; fewer for
                                     wide windows) and lanes / walkers per block are not forced, else the chain
                                     form), REWL_SWEEP_CHAIN (32 lanes: the warp decides 32 trials together and
                                     makes its own draws; fewer lanes: two-deep chain), REWL_SWEEP_STAGED (staged

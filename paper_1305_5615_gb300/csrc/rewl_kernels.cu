@@ -950,7 +950,7 @@ __global__ void __launch_bounds__(32 * kResolveWarps, 12) k_sweep_resolve(Proble
 }
 
 // One walker a CTA, its draws made by further warps.
-constexpr int kRingCtas = 7;  // that an SM's registers hold (97 a thread)
+constexpr int kRingCtas = 6;  // that an SM's registers hold (113 a thread; 7 need spills: Potts q = 10, 512 walkers 22.1 ms, with 6 20.6)
 template <int MODEL>
 __global__ void __launch_bounds__(kRingThreads, kRingCtas) k_sweep_resolve_ring(Problem P, DevState S, SweepLaunch A) {
   sweep_resolve_ring_body<MODEL>(P, S, A.n_att, S.active[blockIdx.x], A.wait_cycles);
@@ -1384,7 +1384,7 @@ bool resolve_fits(const Problem& P, int wpb) { return resolve_smem_bytes(P, wpb,
 size_t resolve_smem(const Problem& P, int wpb, bool ring) { return resolve_smem_bytes(P, wpb, ring); }
 
 // Walkers an SM runs at once in the ring form.  Up to there the ring form is the faster one (Ising 32 x 32, ln f =
-// 2^-18, 1024 walkers: 64 cycles a trial against 76 with the draws in the same warp; 64 walkers: 41 against 59);
+// 2^-18, 512 walkers: 50 cycles a trial against 63 with the draws in the same warp; 64 walkers: 41 against 59);
 // a second wave of CTAs would double its time (1280 walkers of Ising 21 x 21: 97 against 90).
 int ring_walkers_per_sm(const Problem& P) {
   return (int)std::min<size_t>(kRingCtas, kMaxSmem / (resolve_smem_bytes(P, 1, true) + 1024));
