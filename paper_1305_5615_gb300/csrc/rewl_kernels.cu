@@ -950,7 +950,9 @@ __global__ void __launch_bounds__(32 * kResolveWarps, 12) k_sweep_resolve(Proble
 }
 
 // One walker a CTA, its draws made by further warps.
-constexpr int kRingCtas = 6;  // that an SM's registers hold (113 a thread; 7 need spills: Potts q = 10, 512 walkers 22.1 ms, with 6 20.6)
+// Asked to fit 7 an SM the compiler takes 80 registers and spills (Potts q = 10, 512 walkers 22.1 ms), asked for 6 it
+// takes 94 - 96 and does not (20.6 ms).
+constexpr int kRingCtas = 6;
 template <int MODEL>
 __global__ void __launch_bounds__(kRingThreads, kRingCtas) k_sweep_resolve_ring(Problem P, DevState S, SweepLaunch A) {
   sweep_resolve_ring_body<MODEL>(P, S, A.n_att, S.active[blockIdx.x], A.wait_cycles);
@@ -1384,10 +1386,26 @@ bool resolve_fits(const Problem& P, int wpb) { return resolve_smem_bytes(P, wpb,
 size_t resolve_smem(const Problem& P, int wpb, bool ring) { return resolve_smem_bytes(P, wpb, ring); }
 
 // Walkers an SM runs at once in the ring form.  Up to there the ring form is the faster one (Ising 32 x 32, ln f =
-// 2^-18, 512 walkers: 50 cycles a trial against 63 with the draws in the same warp; 64 walkers: 41 against 59);
-// a second wave of CTAs would double its time (1280 walkers of Ising 21 x 21: 97 against 90).
+// 2^-18, 512 walkers: 50 cycles a trial against 63 with the draws in the same warp; 64 walkers: 41 against 59;
+// 912, six an SM: 84 against 83); a second wave of CTAs would double its time.
+template <int MODEL>
+static int ring_walkers_per_sm_m(size_t smem) {
+  int n = 0;
+  if (cudaFuncSetAttribute(k_sweep_resolve_ring<MODEL>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_sweep_resolve_ring<MODEL>, kRingThreads, smem) != cudaSuccess)
+    n = 0;
+  return n;
+}
 int ring_walkers_per_sm(const Problem& P) {
-  return (int)std::min<size_t>(kRingCtas, kMaxSmem / (resolve_smem_bytes(P, 1, true) + 1024));
+  const size_t smem = resolve_smem_bytes(P, 1, true);
+  if (smem > kMaxSmem) return 0;
+  switch (P.model) {
+    case kIsing: return ring_walkers_per_sm_m<kIsing>(smem);
+    case kPotts: return ring_walkers_per_sm_m<kPotts>(smem);
+    case kEA: return ring_walkers_per_sm_m<kEA>(smem);
+    case kEA3: return ring_walkers_per_sm_m<kEA3>(smem);
+  }
+  return 0;
 }
 
 template <int MODEL, int G>
