@@ -66,7 +66,7 @@ N_SM = 152
 PROFILE_SUMMARY = os.path.join(ROOT, "profiles", "k_sweep_ising_L32_h16_m4.txt")
 
 
-SWEEP_SOURCES = ("rewl_device.cuh", "rewl_kernels.cu", "rewl_layout.h")
+SWEEP_SOURCES = ("rewl_device.cuh", "rewl_kernels.cu", "rewl_layout.h", "rewl_resolve.cuh")
 
 
 def kernel_source_hash():
@@ -518,7 +518,8 @@ def run_gb300(args, wl, world, rank, local):
         rate = measured_int_rate()
         peak = N_SM * (rate or 128.0) * f_max / 1e12
         traffic = traffic_from_profile(args.workload, i1["sweep_variant"])
-        names = {0: "k_sweep_chain", 1: "k_sweep_spec", 2: "k_sweep_ring"}
+        names = {0: "k_sweep_resolve" if i1["lanes_per_walker"] == 32 else "k_sweep_chain", 1: "k_sweep_spec",
+                 2: "k_sweep_resolve_ring"}
         roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Tops/s", "frac": achieved / peak,
                 "traffic": traffic, "kernel": names.get(i1["sweep_variant"], "k_sweep"), "avg_launch_ms": avg_s * 1e3,
                 "attempts_per_launch": att_per_launch, "ops_per_attempt": OPS_PER_ATTEMPT,
@@ -540,7 +541,9 @@ def run_gb300(args, wl, world, rank, local):
                                "frac": iso / cyc, "sm_mhz": f_run, "walkers": walkers,
                                "chain_bound_attempts_per_s": walkers * f_run * 1e6 / iso,
                                "basis": "the sequential WL step alone (dependency chain only), measured by "
-                                        "ubench/rates.cu on the GB300; bound = walkers x SM clock / its cycles"}
+                                        "ubench/rates.cu on the GB300; bound = walkers x SM clock / its cycles.  "
+                                        "The default forms decide 32 trials together and are not held by it: frac "
+                                        "says how many times faster than one trial after the other they are"}
 
     cpu = None
     if rank == 0 and world == 1 and not args.no_cpu:
@@ -578,7 +581,7 @@ def run_gb300(args, wl, world, rank, local):
                                                    "ms_per_launch")} for r in tune_res]) if tune_res else
                            "automatic (sweep_variant %d)" % i1["sweep_variant"]},
                 "roofline": roof, "cpu_baseline": cpu, "e2e": e2e,
-                "gpu_launches": args.steps * (3 * (SPF // SPE) + 1), "clocks": clocks,
+                "gpu_launches": args.steps * (2 * (SPF // SPE) + 1), "clocks": clocks,
                 "solve_state": {"sweep_clock": i1["sweep_clock"], "windows_done": i1["windows_done"]},
                 "time_to_dos": tdos}
         print(json.dumps(line), flush=True)

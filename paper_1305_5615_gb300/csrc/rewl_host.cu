@@ -128,15 +128,16 @@ static bool is_pow2_double(double v) {
   return m == 0.5;
 }
 
-// Kernel configuration: G lanes per walker and walkers per CTA.  Few walkers
-// run latency-bound (one sequential chain each), so they get whole warps and
-// are spread over all SMs; many walkers share warps.
+// Kernel configuration: G lanes per walker and walkers per CTA.  A whole warp a
+// walker wherever the forms that decide 32 trials together fit (4096 walkers of
+// Ising 128 x 128: 169 ms against 603 with 8 lanes); few walkers are spread over
+// all SMs.  Only windows too wide for those forms share warps.
 static void choose_config(rewl_ctx* c, int n_sm) {
   const Problem& P = c->P;
   int G = c->params.lanes_per_walker;
   if (G == 0) {
     const int nw = P.n_walkers;
-    if (nw <= ring_walkers_per_sm(P) * n_sm || (c->params.sweep_variant == kSweepChain && resolve_smem(P, 1, false) <= 227 * 1024)) G = 32;
+    if (nw <= 8 * n_sm || (c->params.sweep_variant == kSweepChain && resolve_smem(P, 1, false) <= 227 * 1024)) G = 32;
     else if (nw <= 32 * n_sm) G = 8;
     else G = 4;
   }
@@ -144,7 +145,7 @@ static void choose_config(rewl_ctx* c, int n_sm) {
   if (wpb == 0 && G == 32 && c->params.sweep_variant == kSweepChain) {
     // warps that decide 32 trials together share nothing but the couplings: two a CTA, so that the 32 CTAs an SM
     // takes are no limit (128 x 128 Ising, 4096 walkers, 10 sweeps: 9.77 ms with one, 9.69 with two, 9.71 with four)
-    wpb = resolve_smem(P, 2, false) <= 100 * 1024 ? 2 : 1;
+    wpb = P.n_walkers > n_sm && resolve_smem(P, 2, false) <= 100 * 1024 ? 2 : 1;
   } else if (wpb == 0) {
     wpb = std::max(1, 256 / G);
     const size_t budget = 200 * 1024;
@@ -488,7 +489,11 @@ rewl_status rewl_create(rewl_handle* out, const rewl_model* model, const rewl_la
   int dev = 0, n_sm = 152;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+  // a few walkers were always charged the ring variant's shared memory, whichever form their window now gets
+  int charged = c->params.sweep_variant;
   if (c->params.sweep_variant == REWL_SWEEP_AUTO) {
+    charged = P.n_walkers <= 8 * n_sm && (prm.lanes_per_walker == 0 || prm.lanes_per_walker == 32) &&
+                      prm.walkers_per_block <= 1 ? kSweepRing : kSweepChain;
     // latency-bound solves (as many walkers as the ring form runs in one wave) get their draws from
     // producer warps; with more walkers each warp makes its own
     const bool own_sm = P.n_walkers <= ring_walkers_per_sm(P) * n_sm && (prm.lanes_per_walker == 0 || prm.lanes_per_walker == 32) &&
@@ -517,9 +522,9 @@ rewl_status rewl_create(rewl_handle* out, const rewl_model* model, const rewl_la
       c->pre_on = true;
     }
   }
-  if (sweep_smem_bytes(P, c->wpb, c->G, c->params.sweep_variant) > 227 * 1024)
+  if (sweep_smem_bytes(P, charged == kSweepRing ? 1 : c->wpb, c->G, charged) > 227 * 1024)
     return bail(fail(REWL_EINVAL, "a walker needs %zu bytes of shared memory (window of %d bins)",
-                     sweep_smem_bytes(P, 1, c->G, c->params.sweep_variant), P.w));
+                     sweep_smem_bytes(P, 1, c->G, charged), P.w));
   st = upload_active(c);
   if (st != REWL_OK) return bail(st);
 #undef BAIL_CUDA
