@@ -115,9 +115,9 @@ typedef struct {
                                     strictly increasing starts and ends, neighbours sharing >= 1 bin */
   const int32_t* window_widths;  /* `windows` widths in bins, with window_starts (both or neither) */
   int64_t wait_cycles;           /* bound of the ring form's hand-off waits between a walker's warp and
-                                    its producer warp, in SM clock cycles from the start of a sweep
+                                    its producer warps, in SM clock cycles from the start of a sweep
                                     launch; 0 = 2^34 (about 8 s at 2 GHz, while a launch takes
-                                    milliseconds).  When a wait runs out both warps stop early and
+                                    milliseconds).  When a wait runs out all of them stop early and
                                     rewl_step returns REWL_ETIMEOUT at its next flatness check */
   int32_t server_walker_target;  /* served form: no request is admitted while at least this many walkers of
                                     windows not yet done are running (the first always is); 0 = 24 per SM,
@@ -288,8 +288,8 @@ rewl_status rewl_get_state(rewl_handle h, rewl_state* st);
 
 /*
  * rewl_autotune -- picks the sweep kernel's launch shape for one problem by
- * timing candidates on the problem itself: the ring form (32 lanes and a
- * producer warp per walker) and the chain form with 32, 16, 8, 4 and 2 lanes
+ * timing candidates on the problem itself: the ring form (32 lanes and two
+ * producer warps per walker) and the chain form with 32, 16, 8, 4 and 2 lanes
  * per walker (walkers per CTA as rewl_create chooses).  Each candidate is a
  * fresh rewl_create with the given arguments, one warm-up block, then `sweeps`
  * sweeps timed with CUDA events around every sweep launch.  All candidates
@@ -398,9 +398,9 @@ rewl_status rewl_thermo_jackknife(const double* lng_runs, int32_t n_runs, int32_
  * would wait for the slowest walker of all).  A group advances by
  * rounds: for every request of the group one block of sweeps_per_exchange
  * sweeps, one exchange round and, when due, the flatness check -- one fused
- * launch for the sweeps of all the group's walkers (with a producer warp per
- * walker while the GPU holds few walkers, else 4 walkers of a request per
- * CTA), one launch each for the exchanges, clocks and flatness checks of all
+ * launch for the sweeps of all the group's walkers (with producer warps for
+ * every walker while the GPU holds few walkers, else one warp per
+ * walker), one launch each for the exchanges, clocks and flatness checks of all
  * its requests.  Every phase boundary is decided on the device (clocks,
  * flatness, merges and done flags are device state; the kernels of finished
  * windows and requests do nothing), so a group's k rounds and the report read

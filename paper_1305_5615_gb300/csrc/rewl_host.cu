@@ -130,7 +130,7 @@ static bool is_pow2_double(double v) {
 
 // Kernel configuration: G lanes per walker and walkers per CTA.  A whole warp a
 // walker wherever the forms that decide 32 trials together fit (4096 walkers of
-// Ising 128 x 128: 169 ms against 603 with 8 lanes); few walkers are spread over
+// Ising 128 x 128, 200 sweeps: 169 - 186 ms against 600 with 8 lanes); few walkers are spread over
 // all SMs.  Only windows too wide for those forms share warps.
 static void choose_config(rewl_ctx* c, int n_sm) {
   const Problem& P = c->P;

@@ -18,13 +18,13 @@
 // (first guess included: all trials judged from the group's first bin), 4.2 on
 // an 8 x 8 lattice, and 5 - 9 at ln f = 1.
 //
-// A pass is a chain of about 225 cycles of a lone warp (340 with counted visits),
+// A pass is a chain of about 225 cycles of a lone warp (333 with counted visits),
 // a group about 530 besides.  Against the sequential forms, 1000 sweeps, whole
-// calls: Ising 32 x 32, 64 walkers, ln f = 2^-18 66.3 -> 15.8 ms (132 -> 31 cycles
-// a trial of a walker), at ln f = 1 67.6 -> 52.9 ms; Potts q = 10 32 x 32, 512
-// walkers 75.0 -> 23.0 ms; +-J 12^3 114 -> 25.7 ms; Ising 8 x 8 to ln f < 1e-6
-// 723 -> 135 ms; and Ising 128 x 128, 4096 walkers, 200 sweeps 603 -> 190 ms,
-// where issue is what bounds it (409 warp instructions a group).
+// calls: Ising 32 x 32, 64 walkers, ln f = 2^-18 66.1 -> 15.7 ms (134 -> 32 cycles
+// a trial of a walker), from ln f = 1 on 67.4 -> 48.6 ms; Potts q = 10 32 x 32, 512
+// walkers 75.1 -> 20.6 ms; +-J 12^3 114 -> 25.0 ms; Ising 8 x 8 to ln f < 1e-6
+// 615 -> 114 ms; and Ising 128 x 128, 4096 walkers, 200 sweeps 600 -> 169 - 186 ms,
+// where issue is what bounds it (371 warp instructions a group).
 //
 // Visits.  ln g of a bin grows by ln f a visit, also inside the group.  For a
 // trial the counts of two bins differ by at most the number of earlier trials,
