@@ -18,13 +18,13 @@
 // (first guess included: all trials judged from the group's first bin), 4.2 on
 // an 8 x 8 lattice, and 5 - 9 at ln f = 1.
 //
-// A pass is a chain of about 225 cycles of a lone warp (333 with counted visits),
+// A pass is a chain of about 225 cycles of a lone warp (320 with counted visits),
 // a group about 530 besides.  Against the sequential forms, 1000 sweeps, whole
-// calls: Ising 32 x 32, 64 walkers, ln f = 2^-18 66.1 -> 15.7 ms (134 -> 32 cycles
-// a trial of a walker), from ln f = 1 on 67.4 -> 48.6 ms; Potts q = 10 32 x 32, 512
-// walkers 75.1 -> 20.6 ms; +-J 12^3 114 -> 25.0 ms; Ising 8 x 8 to ln f < 1e-6
-// 615 -> 114 ms; and Ising 128 x 128, 4096 walkers, 200 sweeps 600 -> 169 - 186 ms,
-// where issue is what bounds it (371 warp instructions a group).
+// calls: Ising 32 x 32, 64 walkers, ln f = 2^-18 66.1 -> 15.6 ms (134 -> 32 cycles
+// a trial of a walker), from ln f = 1 on 67.4 -> 47.0 ms; Potts q = 10 32 x 32, 512
+// walkers 75.1 -> 20.6 ms; +-J 12^3 114 -> 24.8 ms; Ising 8 x 8 to ln f < 1e-6
+// 615 -> 112 ms; and Ising 128 x 128, 4096 walkers, 200 sweeps 600 -> 169 - 186 ms,
+// where issue is what bounds it (385 warp instructions a group).
 //
 // Visits.  ln g of a bin grows by ln f a visit, also inside the group.  For a
 // trial the counts of two bins differ by at most the number of earlier trials,
@@ -247,7 +247,9 @@ __host__ __device__ __forceinline__ int resolve_reach(const Problem& P) {
 // bit; the lanes equal to x are those that agree in every bit.  kBinBits bits hold -16 .. 15, where nearly every
 // group stays; the rest takes eight, which is exact, since the bins of one pass span at most 33 offsets (132 for
 // Potts).  Against a table of lane masks in shared memory (an atomic a trial, many of them on one word): 475 -> 333
-// cycles a pass.
+// cycles a pass.  A bit of x picks the ballot or its complement (a predicate, in place of a mask made of two shifts:
+// Ising 32 x 32 from ln f = 1 on 48.4 -> 47.0 ms
+// with the checks below made once a group and one population count a bond).
 constexpr int kBinBits = 5;
 template <int BITS>
 struct BinMasks {
@@ -256,10 +258,9 @@ struct BinMasks {
 #pragma unroll
     for (int k = 0; k < BITS; ++k) b[k] = __ballot_sync(0xffffffffu, (end >> k) & 1);
   }
-  __device__ __forceinline__ uint32_t equal(int x) const {
-    uint32_t m = 0xffffffffu;
+  __device__ __forceinline__ uint32_t equal(int x, uint32_t m) const {  // of the lanes m
 #pragma unroll
-    for (int k = 0; k < BITS; ++k) m &= b[k] ^ (uint32_t)((int)(~x << (31 - k)) >> 31);
+    for (int k = 0; k < BITS; ++k) m &= (x >> k) & 1 ? b[k] : ~b[k];
     return m;
   }
 };
@@ -536,10 +537,9 @@ __device__ __forceinline__ void resolve_walker(const Problem& P, const DevState&
       off.cut(d, 0u);
     } else {
       uint32_t bonds = sat;  // every accepted flip of the site turns all its bonds, one of a neighbour the bond to it
-      if constexpr (kMasks) {
-        bonds ^= (__popc(A & h.s) & 1) ? kAll : 0u;
+      if constexpr (kMasks) {  // a trial is at the site or at a neighbour, not at both: one count a bond
 #pragma unroll
-        for (int k = 0; k < NB; ++k) bonds ^= (__popc(A & h.n[k]) & 1u) << k;
+        for (int k = 0; k < NB; ++k) bonds ^= (__popc(A & (h.s ^ h.n[k])) & 1u) << k;
       } else {
         const uint32_t on1 = __funnelshift_r(A, 0u, aux >> 6) & 1u, on2 = __funnelshift_r(A, 0u, aux >> 11) & 1u;
         bonds ^= on1 * ((aux >> 16) & kAll) ^ on2 * ((aux >> 22) & kAll);
@@ -553,7 +553,7 @@ __device__ __forceinline__ void resolve_walker(const Problem& P, const DevState&
   int64_t gap = 0, f_old = 0, f_new = 0;  // gap: ln g(old) - ln g(new) - ln u
   int v_old = 0, v_new = 0;
   bool inwin = true;
-  auto pass = [&](auto bin_bits, uint32_t& wide) -> uint32_t {
+  auto pass = [&](auto bin_bits, bool& wide) -> uint32_t {
     constexpr int BITS = decltype(bin_bits)::value;
     const int rel = off.sum(A & lt), to = rel + d;  // bins from the group's first
     at = bin + rel;
@@ -564,10 +564,11 @@ __device__ __forceinline__ void resolve_walker(const Problem& P, const DevState&
     if constexpr (BITS > 0) {
       const int end = (A & bit) ? to : rel;
       const BinMasks<BITS> ends(end);
-      // the bins asked for are at most 4 further than the end bins
-      if constexpr (BITS < 8) wide = __ballot_sync(0xffffffffu, (uint32_t)(end + (1 << (BITS - 1)) - 4) >= (1u << BITS) - 8u);
-      v_old = __popc(ends.equal(rel) & lt);
-      v_new = __popc(ends.equal(to) & lt);
+      // the bins asked for are at most kMaxOffset further than the end bins
+      constexpr uint32_t kFar = kMaxOffset<MODEL>;
+      if constexpr (BITS < 8) wide = (uint32_t)end + (1u << (BITS - 1)) - kFar >= (1u << BITS) - 2u * kFar;
+      v_old = __popc(ends.equal(rel, lt));
+      v_new = __popc(ends.equal(to, lt));
       gap += (int64_t)(v_old - v_new) << lsh;
     }
     return __ballot_sync(0xffffffffu, inwin && gap >= 0);
@@ -577,8 +578,7 @@ __device__ __forceinline__ void resolve_walker(const Problem& P, const DevState&
     uint32_t fixed = 0u, value = 0u;  // trials decided in FP64, and their decisions
     if constexpr (!DENSE) load_masks(g);
     while (true) {
-      bool again;
-      uint32_t wide;
+      bool again, wide;
       do {
         const uint32_t was = nv;
         offset(std::true_type{});
@@ -612,7 +612,9 @@ __device__ __forceinline__ void resolve_walker(const Problem& P, const DevState&
     atomicXor(&M.lat[site], (acc ? (MODEL == kPotts ? v ^ nv : 1u) : 0u) << shift);
     post = acc ? at + d : at;
     counting = n_att - g * 32u >= 32u ? 0xffffffffu : (1u << (n_att - g * 32u)) - 1u;
-    bin = __shfl_sync(0xffffffffu, post, 31);
+    // the sum does not wait for `post`; with own draws (bound by issue) and with Potts' four bits a shuffle is less
+    if constexpr (RING && MODEL != kPotts) bin += off.sum(A);
+    else bin = __shfl_sync(0xffffffffu, post, 31);
     n_acc += acc;
     __syncwarp();
     if constexpr (RING) ring->release(g, lane);
@@ -688,11 +690,13 @@ __device__ __forceinline__ void resolve_walker(const Problem& P, const DevState&
       // a trial this close to the line is told by `settle` alone: without counted visits, closer than one ln f for
       // every earlier trial
       const uint32_t margin = COUNT ? 1u : clear_24;
-      auto too_close = [&]() { return __ballot_sync(0xffffffffu, inwin && (uint32_t)(gap >> 24) + margin < 2u * margin + 1u); };
-      bool again = true;
+      auto too_close = [&](bool or_else) {
+        return __ballot_sync(0xffffffffu, or_else || (inwin && (uint32_t)(gap >> 24) + margin < 2u * margin + 1u));
+      };
+      bool again = true, wide = false;
       if constexpr (!RING) off.cut(d, sat);
       if constexpr (!RING && !COUNT) {
-        leave = too_close();
+        leave = too_close(false);
         // a guess without a move or a touched neighbourhood is the fixed point
         again = __any_sync(0xffffffffu, (A & bit) != 0u && (d != 0 || (touched & bit) != 0u));
       }
@@ -704,14 +708,16 @@ __device__ __forceinline__ void resolve_walker(const Problem& P, const DevState&
         if (RING || touched) offset(Masks{});
         const bool moved = MODEL == kPotts && __any_sync(0xffffffffu, nv != was);  // proposed values others may build on
         do {
-          uint32_t wide = 0u;
           const uint32_t B = pass(std::integral_constant<int, COUNT ? kBinBits : 0>{}, wide);
-          leave = too_close() | wide;
+          if constexpr (!COUNT) leave = too_close(false);
           again = B != A;
           A = B;
         } while (!kEachPass && again && (A & touched) == by);
         again = again || moved;
       }
+      // With counted visits (many passes) the checks are made once, of the settled pass: bins that kBinBits do not
+      // hold make a pass's decisions wrong, but still depend on the trials before alone, so the passes end.
+      if constexpr (COUNT) leave = too_close(wide);
       if constexpr (!DENSE) leave |= aux >> 31;
       if (leave != 0u) break;
       commit(g);
