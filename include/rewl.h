@@ -99,13 +99,17 @@ typedef struct {
                                     ring form when its CTAs, one a walker, run in one wave (6 per SM; fewer for
                                     wide windows) and lanes / walkers per block are not forced, else the chain
                                     form), REWL_SWEEP_CHAIN (32 lanes: the warp decides 32 trials together and
-                                    makes its own draws; fewer lanes: two-deep chain), REWL_SWEEP_STAGED (staged
-                                    one-deep chain), REWL_SWEEP_RING (32 trials decided together, draws made by
-                                    producer warps of the CTA; 32 lanes and one walker per CTA) */
-  int32_t prefetch_draws;        /* 1 = in plain mode with variant 0 the draws of the next block (sites,
-                                    ln u, conflict masks) are prepared on a second stream while the current
-                                    block runs, when both buffers fit in 1 GiB; 0 = no (default: kernels
-                                    running beside the sweep slow its chains) */
+                                    makes its own draws, unless prefetch_draws applies; else two-deep chain),
+                                    REWL_SWEEP_STAGED (staged one-deep chain), REWL_SWEEP_RING (32 trials
+                                    decided together, draws made by producer warps of the CTA; 32 lanes and
+                                    one walker per CTA) */
+  int32_t prefetch_draws;        /* 1 = in plain mode, for the sequential chain form (variant 0 asked for, or
+                                    taken because the window is too wide for the forms that decide 32
+                                    trials together; at least 8 lanes), the draws of a block (sites, ln u,
+                                    conflict masks) are prepared by a kernel ahead of its sweeps, when they
+                                    fit in 512 MiB.  The sweeps then take their trials one after the other,
+                                    also with 32 lanes: several times slower than the default forms;
+                                    0 = no (default) */
   int32_t wl_rule;               /* how ln f falls (the WL "update/convergence rule"): REWL_RULE_FLAT or
                                     REWL_RULE_ONE_OVER_T; see below */
   const int32_t* window_starts;  /* NULL: the equal partition of Fig. 1a from `windows` and `overlap`.
@@ -230,7 +234,7 @@ typedef struct {
   double sweep_ms;           /* their summed device time, CUDA events on the solve's stream */
   int64_t h2d_bytes;         /* bytes copied host -> device by this handle so far */
   int64_t d2h_bytes;         /* bytes copied device -> host by this handle so far */
-  int32_t prefetch_draws;    /* 1 when the next block's draws are prepared on a second stream */
+  int32_t prefetch_draws;    /* 1 when a block's draws are prepared ahead of its sweeps */
   int32_t sweep_variant;     /* the sweep form in use (REWL_SWEEP_CHAIN, _STAGED or _RING) */
 } rewl_info;
 

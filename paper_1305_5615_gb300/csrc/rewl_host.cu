@@ -66,14 +66,8 @@ rewl_ctx::~rewl_ctx() {
     if (params.free) params.free(p, (void*)stream, params.alloc_user);
     else cudaFree(p);
   }
-  if (pre_stream) cudaStreamSynchronize(pre_stream);
   if (h_n_done) cudaFreeHost(h_n_done);
   for (cudaEvent_t e : ev_pool) cudaEventDestroy(e);
-  for (int k = 0; k < 2; ++k) {
-    if (ev_pre[k]) cudaEventDestroy(ev_pre[k]);
-    if (ev_used[k]) cudaEventDestroy(ev_used[k]);
-  }
-  if (pre_stream) cudaStreamDestroy(pre_stream);
   if (own_stream && stream) cudaStreamDestroy(stream);
 }
 
@@ -131,13 +125,17 @@ static bool is_pow2_double(double v) {
 // Kernel configuration: G lanes per walker and walkers per CTA.  A whole warp a
 // walker wherever the forms that decide 32 trials together fit (4096 walkers of
 // Ising 128 x 128, 200 sweeps: 169 - 186 ms against 600 with 8 lanes); few walkers are spread over
-// all SMs.  Only windows too wide for those forms share warps.
+// all SMs.  Only windows too wide for those forms share warps, and prepared draws, which those forms do not take:
+// a whole warp up to 12 walkers an SM (1000 sweeps of 16 x 16, 1280 walkers: Ising 49 ms against 63 with 8 lanes,
+// Potts q = 10 52 against 64; 12 x 12, 2048 walkers: 40 against 40, 44 against 40).
 static void choose_config(rewl_ctx* c, int n_sm) {
   const Problem& P = c->P;
+  const int nw = P.n_walkers;
   int G = c->params.lanes_per_walker;
   if (G == 0) {
-    const int nw = P.n_walkers;
-    if (nw <= 8 * n_sm || (c->params.sweep_variant == kSweepChain && resolve_smem(P, 1, false) <= 227 * 1024)) G = 32;
+    const bool warp = c->pre_on ? nw <= 12 * n_sm && sweep_smem_bytes(P, 2, 32, kSweepChain) <= 100 * 1024
+                                : c->params.sweep_variant == kSweepChain && resolve_smem(P, 1, false) <= 227 * 1024;
+    if (nw <= 8 * n_sm || warp) G = 32;
     else if (nw <= 32 * n_sm) G = 8;
     else G = 4;
   }
@@ -145,12 +143,12 @@ static void choose_config(rewl_ctx* c, int n_sm) {
   if (wpb == 0 && G == 32 && c->params.sweep_variant == kSweepChain) {
     // warps that decide 32 trials together share nothing but the couplings: two a CTA, so that the 32 CTAs an SM
     // takes are no limit (128 x 128 Ising, 4096 walkers, 10 sweeps: 9.77 ms with one, 9.69 with two, 9.71 with four)
-    wpb = P.n_walkers > n_sm && resolve_smem(P, 2, false) <= 100 * 1024 ? 2 : 1;
+    wpb = nw > n_sm && resolve_smem(P, 2, false) <= 100 * 1024 ? 2 : 1;
   } else if (wpb == 0) {
     wpb = std::max(1, 256 / G);
     const size_t budget = 200 * 1024;
     while (wpb > 1 && sweep_smem_bytes(P, wpb, G, c->params.sweep_variant) > budget) --wpb;
-    const int spread = (P.n_walkers + n_sm - 1) / n_sm;  // at least one CTA per SM when possible
+    const int spread = (nw + n_sm - 1) / n_sm;  // at least one CTA per SM when possible
     wpb = std::max(1, std::min(wpb, spread));
   }
   wpb = std::max(1, std::min(wpb, 256 / G));
@@ -500,27 +498,22 @@ rewl_status rewl_create(rewl_handle* out, const rewl_model* model, const rewl_la
                         prm.walkers_per_block <= 1;
     c->params.sweep_variant = own_sm ? kSweepRing : kSweepChain;
   }
+  // Draws prepared by a kernel of their own ahead of each block's sweeps: plain mode, chain variant with at least 8
+  // lanes, within 512 MiB; not where the automatic choice has a form that decides 32 trials together, which is the
+  // faster one (Ising 16 x 16, 1000 sweeps, 1000 walkers 18 ms against 41 with prepared draws).
+  const uint64_t pre_stride = ((uint64_t)prm.sweeps_per_exchange * P.N + 31) / 32 * 32;
+  const uint64_t pre_bytes = (uint64_t)P.n_walkers * pre_stride * sizeof(PreTrial);
+  const int lanes = prm.lanes_per_walker;
+  c->pre_on = prm.prefetch_draws == 1 && prm.mode == REWL_MODE_PLAIN && c->params.sweep_variant == kSweepChain &&
+              pre_bytes <= (512ull << 20) && (lanes ? lanes >= 8 : P.n_walkers <= 32 * n_sm) &&
+              (prm.sweep_variant != REWL_SWEEP_AUTO || (lanes != 0 && lanes != 32) || resolve_smem(P, 1, false) > 227 * 1024);
   choose_config(c, n_sm);
   c->n_sm = n_sm;
   BAIL_CUDA(prepare_sweep(c->G, P.model));
-  // Draws prepared ahead on the idle SMs: plain mode, chain kernel, G >= 8, both buffers within 1 GiB.
-  {
-    const uint64_t n_att = (uint64_t)prm.sweeps_per_exchange * P.N;
-    const uint64_t stride = (n_att + 31) / 32 * 32;
-    const uint64_t bytes = (uint64_t)P.n_walkers * stride * sizeof(PreTrial);
-    if (prm.prefetch_draws == 1 && prm.mode == REWL_MODE_PLAIN && c->params.sweep_variant == kSweepChain && c->G >= 8 &&
-        2 * bytes <= (1ull << 30)) {
-      c->pre_stride = (uint32_t)stride;
-      c->pre_buf[0] = (PreTrial*)c->dalloc(bytes, &st);
-      c->pre_buf[1] = (PreTrial*)c->dalloc(bytes, &st);
-      if (st != REWL_OK) return bail(st);
-      BAIL_CUDA(cudaStreamCreateWithFlags(&c->pre_stream, cudaStreamNonBlocking));
-      for (int k = 0; k < 2; ++k) {
-        BAIL_CUDA(cudaEventCreateWithFlags(&c->ev_pre[k], cudaEventDisableTiming));
-        BAIL_CUDA(cudaEventCreateWithFlags(&c->ev_used[k], cudaEventDisableTiming));
-      }
-      c->pre_on = true;
-    }
+  if (c->pre_on) {
+    c->pre_stride = (uint32_t)pre_stride;
+    c->pre_buf = (PreTrial*)c->dalloc(pre_bytes, &st);
+    if (st != REWL_OK) return bail(st);
   }
   if (sweep_smem_bytes(P, charged == kSweepRing ? 1 : c->wpb, c->G, charged) > 227 * 1024)
     return bail(fail(REWL_EINVAL, "a walker needs %zu bytes of shared memory (window of %d bins)",
@@ -534,8 +527,6 @@ rewl_status rewl_create(rewl_handle* out, const rewl_model* model, const rewl_la
 
 void rewl_destroy(rewl_handle h) { delete h; }
 
-static bool with_graph_capture(const rewl_ctx* c) { return c->params.mode == REWL_MODE_GRAPH; }
-
 // One block: sweeps, exchange, clock advance; plus the flatness check when due.
 static rewl_status enqueue_block(rewl_ctx* c, bool with_flat) {
   SweepLaunch A{};
@@ -544,18 +535,13 @@ static rewl_status enqueue_block(rewl_ctx* c, bool with_flat) {
   A.wpb = c->wpb;
   A.variant = c->params.sweep_variant;
   A.wait_cycles = c->params.wait_cycles > 0 ? c->params.wait_cycles : kDefaultWaitCycles;
-  if (c->pre_on && !with_graph_capture(c)) {
-    // this block's draws: prepared by the previous block (checked by its first trial index), else now
-    const uint64_t t0 = c->sweep_clock * (uint64_t)c->P.N;
-    const int k = c->pre_cur;
-    if (c->pre_t0[k] != t0) {
-      CUDA_TRY(cudaStreamWaitEvent(c->pre_stream, c->ev_used[k], 0));
-      CUDA_TRY(launch_precompute(c->G, c->P, t0, A.n_att, c->pre_stride, c->pre_buf[k], c->n_sm, c->pre_stream));
-      CUDA_TRY(cudaEventRecord(c->ev_pre[k], c->pre_stream));
-      c->pre_t0[k] = t0;
-    }
-    CUDA_TRY(cudaStreamWaitEvent(c->stream, c->ev_pre[k], 0));
-    A.pre = c->pre_buf[k];
+  if (c->pre_on) {
+    // Ahead of the sweeps and on their stream: beside them, on a second stream, the kernel's CTAs could be placed first
+    // and then the walkers' CTAs share SMs for the whole launch (Ising 32 x 32, 64 walkers, 1000 sweeps: 108 - 177 ms,
+    // this way 80; where the two overlapped well this costs 1 - 3%).
+    CUDA_TRY(launch_precompute(c->G, c->P, c->sweep_clock * (uint64_t)c->P.N, A.n_att, c->pre_stride, c->pre_buf,
+                               c->n_sm, c->stream));
+    A.pre = c->pre_buf;
     A.pre_stride = c->pre_stride;
   }
   const bool timed = c->params.profile && c->params.mode == REWL_MODE_PLAIN;
@@ -571,17 +557,6 @@ static rewl_status enqueue_block(rewl_ctx* c, bool with_flat) {
   }
   CUDA_TRY(launch_sweep(c->G, c->P, c->S, A, c->stream));
   if (timed) CUDA_TRY(cudaEventRecord(c->ev_pool[2 * c->ev_pending++ + 1], c->stream));
-  if (A.pre) {
-    // the next block's draws go into the other buffer while this block runs
-    const int k = c->pre_cur, k2 = k ^ 1;
-    const uint64_t t0n = (c->sweep_clock + (uint64_t)c->params.sweeps_per_exchange) * (uint64_t)c->P.N;
-    CUDA_TRY(cudaEventRecord(c->ev_used[k], c->stream));
-    CUDA_TRY(cudaStreamWaitEvent(c->pre_stream, c->ev_used[k2], 0));
-    CUDA_TRY(launch_precompute(c->G, c->P, t0n, A.n_att, c->pre_stride, c->pre_buf[k2], c->n_sm, c->pre_stream));
-    CUDA_TRY(cudaEventRecord(c->ev_pre[k2], c->pre_stream));
-    c->pre_t0[k2] = t0n;
-    c->pre_cur = k2;
-  }
   CUDA_TRY(launch_exchange(c->P, c->S, (uint32_t)c->params.sweeps_per_exchange, c->stream));
   if (with_flat) CUDA_TRY(launch_flat_merge(c->P, c->S, c->stream));
   return REWL_OK;

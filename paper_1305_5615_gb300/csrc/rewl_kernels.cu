@@ -966,15 +966,12 @@ __global__ void __launch_bounds__(256, 1) k_sweep_chain(Problem P, DevState S, S
 }
 
 // ---------------------------------------------------------------------------
-// Draws of the next sweep launch, prepared while the current one runs (on the
-// SMs the walkers leave idle): for trial i of walker W the site, the proposed
-// Potts offset, ln u, and the conflict mask of its group of G trials -- the
-// same values the sweep kernel would compute, so the results are unchanged.
-// One thread per (walker, trial) in a grid-stride loop over a small grid (one
-// CTA per SM): a grid of thousands of CTAs that starts before the sweep
-// kernel's CTAs are placed would hold the SMs and pack the walkers' CTAs onto
-// few SMs when they free up.  Trials are padded to a multiple of 32, so every
-// warp is wholly in range or wholly out of it.
+// Draws of a sweep launch, prepared ahead of it: for trial i of walker W the
+// site, the proposed Potts offset, ln u, and the conflict mask of its group of
+// G trials -- the same values the sweep kernel would compute, so the results
+// are unchanged.  One thread per (walker, trial) in a grid-stride loop over
+// eight CTAs an SM, which fill it.  Trials are padded to a multiple of 32, so
+// every warp is wholly in range or wholly out of it.
 // ---------------------------------------------------------------------------
 template <int MODEL, int G>
 __global__ void __launch_bounds__(256) k_precompute(Problem P, uint64_t t0, uint32_t n_att, uint32_t stride,
@@ -1009,9 +1006,9 @@ static cudaError_t launch_precompute_m(int G, const Problem& P, uint64_t t0, uin
 }
 
 cudaError_t launch_precompute(int G, const Problem& P, uint64_t t0, uint32_t n_att, uint32_t stride, PreTrial* out,
-                              int max_blocks, cudaStream_t st) {
+                              int n_sm, cudaStream_t st) {
   const uint64_t threads = (uint64_t)P.n_walkers * stride;
-  const unsigned blocks = (unsigned)std::min<uint64_t>((threads + 255) / 256, (uint64_t)std::max(1, max_blocks));
+  const unsigned blocks = (unsigned)std::min<uint64_t>((threads + 255) / 256, 8ull * (uint64_t)n_sm);
   switch (P.model) {
     case kIsing: return launch_precompute_m<kIsing>(G, P, t0, n_att, stride, out, blocks, st);
     case kPotts: return launch_precompute_m<kPotts>(G, P, t0, n_att, stride, out, blocks, st);

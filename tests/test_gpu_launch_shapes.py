@@ -1,0 +1,57 @@
+"""Which form a solve runs in and with which launch shape, where an option or a
+forced shape meets the automatic choice; the states are the same bits in every
+form."""
+import numpy as np
+import pytest
+
+from paper_1305_5615_gb300 import rewl
+
+pytestmark = pytest.mark.gpu
+
+
+def n_sm():
+    import torch
+
+    return torch.cuda.get_device_properties(0).multi_processor_count
+
+
+def same_states(A, B):
+    a, b = A.state(), B.state()
+    for k in ("lattice", "E", "H", "lnf", "iteration", "wl_accept", "x_accepted"):
+        assert np.array_equal(a[k], b[k]), k
+    assert np.array_equal(a["lng"].view(np.uint64), b["lng"].view(np.uint64))
+
+
+@pytest.mark.parametrize("per_sm,variant,lanes,expect", [
+    (7, -1, 0, (0, 32, 0)),    # automatic: the form that decides 32 trials together, which takes no prepared draws
+    (9, -1, 0, (0, 32, 0)),
+    (9, -1, 8, (0, 8, 1)),     # lanes that only the sequential chain has
+    (9, 0, 0, (0, 32, 1)),     # the chain asked for: prepared draws, a whole warp up to 12 walkers an SM
+    (13, 0, 0, (0, 8, 1)),
+    (33, 0, 0, (0, 32, 0)),    # too many walkers for prepared draws
+])
+def test_prepared_draws_leave_the_faster_forms_alone(per_sm, variant, lanes, expect):
+    m = -(-per_sm * n_sm() // 4)
+    kw = dict(lanes_per_walker=lanes, sweeps_per_exchange=20, sweeps_per_flat_check=100)
+    A = rewl.REWL("ising", 8, 4, 0.75, m, 0.8, 1e-8, 5, sweep_variant=variant, prefetch_draws=1, **kw)
+    got = A.info["sweep_variant"], A.info["lanes_per_walker"], A.info["prefetch_draws"]
+    assert got == expect
+    B = rewl.REWL("ising", 8, 4, 0.75, m, 0.8, 1e-8, 5, sweep_variant=1, **kw)
+    for D in (A, B):
+        D.step(200)
+    same_states(A, B)
+
+
+def test_sweeps_with_prepared_draws_take_as_long_queued_as_one_at_a_time():
+    """Ten blocks queued back to back against blocks waited for one by one: the kernel that prepares draws does not
+    take the sweeps' places on the chip (it once doubled their time; the bound leaves room for the walk itself)."""
+    D = rewl.REWL("ising", 32, 16, 0.75, 4, 0.8, 1e-8, 5, sweep_variant=0, prefetch_draws=1, profile=True)
+    assert D.info["prefetch_draws"] == 1
+    D.step(100)
+    t0 = D.info["sweep_ms"]
+    for _ in range(9):
+        D.step(100)
+    t1 = D.info["sweep_ms"]
+    D.step(1000)
+    one, queued = (t1 - t0) / 9, (D.info["sweep_ms"] - t1) / 10
+    assert queued < 1.3 * one, (one, queued)
