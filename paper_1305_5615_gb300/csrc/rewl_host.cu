@@ -122,42 +122,51 @@ static bool is_pow2_double(double v) {
   return m == 0.5;
 }
 
-// Kernel configuration: G lanes per walker and walkers per CTA.  A whole warp a
-// walker wherever the forms that decide 32 trials together fit (4096 walkers of
-// Ising 128 x 128, 200 sweeps: 169 - 186 ms against 600 with 8 lanes); few walkers are spread over
-// all SMs.  Only windows too wide for those forms share warps, and prepared draws, which those forms do not take:
-// a whole warp up to 12 walkers an SM (1000 sweeps of 16 x 16, 1280 walkers: Ising 49 ms against 63 with 8 lanes,
-// Potts q = 10 52 against 64; 12 x 12, 2048 walkers: 40 against 40, 44 against 40).
-static void choose_config(rewl_ctx* c, int n_sm) {
-  const Problem& P = c->P;
+// Launch shape of the forms that take a walker's trials one after the other: G lanes a walker, wpb walkers a CTA.
+// Few walkers run latency-bound (one sequential chain each), so they get whole warps and are spread over all SMs; many
+// walkers share warps.  A solve is accepted by this shape's shared memory, whichever form then runs.
+struct LaunchShape {
+  int G, wpb;
+};
+static LaunchShape sequential_shape(const Problem& P, const rewl_params& prm, int variant, int n_sm) {
+  if (variant == kSweepRing) return {32, 1};
   const int nw = P.n_walkers;
-  int G = c->params.lanes_per_walker;
-  if (G == 0) {
-    const bool warp = c->pre_on ? nw <= 12 * n_sm && sweep_smem_bytes(P, 2, 32, kSweepChain) <= 100 * 1024
-                                : c->params.sweep_variant == kSweepChain && resolve_smem(P, 1, false) <= 227 * 1024;
-    if (nw <= 8 * n_sm || warp) G = 32;
-    else if (nw <= 32 * n_sm) G = 8;
-    else G = 4;
-  }
-  int wpb = c->params.walkers_per_block;
-  if (wpb == 0 && G == 32 && c->params.sweep_variant == kSweepChain) {
-    // warps that decide 32 trials together share nothing but the couplings: two a CTA, so that the 32 CTAs an SM
-    // takes are no limit (128 x 128 Ising, 4096 walkers, 10 sweeps: 9.77 ms with one, 9.69 with two, 9.71 with four)
-    wpb = nw > n_sm && resolve_smem(P, 2, false) <= 100 * 1024 ? 2 : 1;
-  } else if (wpb == 0) {
+  const int G = prm.lanes_per_walker ? prm.lanes_per_walker : nw <= 8 * n_sm ? 32 : nw <= 32 * n_sm ? 8 : 4;
+  int wpb = prm.walkers_per_block;
+  if (wpb == 0) {
     wpb = std::max(1, 256 / G);
     const size_t budget = 200 * 1024;
-    while (wpb > 1 && sweep_smem_bytes(P, wpb, G, c->params.sweep_variant) > budget) --wpb;
+    while (wpb > 1 && sweep_smem_bytes(P, wpb, G, variant) > budget) --wpb;
     const int spread = (nw + n_sm - 1) / n_sm;  // at least one CTA per SM when possible
     wpb = std::max(1, std::min(wpb, spread));
   }
-  wpb = std::max(1, std::min(wpb, 256 / G));
-  if (c->params.sweep_variant == kSweepRing) {  // one walker per CTA on a whole warp, plus its producer warp
-    G = 32;
-    wpb = 1;
+  return {G, std::max(1, std::min(wpb, 256 / G))};
+}
+
+// The shape that runs.  A whole warp a walker wherever the forms that decide 32 trials together fit (4096 walkers of
+// Ising 128 x 128, 200 sweeps: 169 - 186 ms against 600 with 8 lanes).  Their warps share nothing but the couplings:
+// two a CTA, so that the 32 CTAs an SM takes are no limit (128 x 128 Ising, 4096 walkers, 10 sweeps: 9.77 ms with one,
+// 9.69 with two, 9.71 with four).  Prepared draws, which those forms do not take: a whole warp up to 12 walkers an SM
+// (1000 sweeps of 16 x 16, 1280 walkers: Ising 49 ms against 63 with 8 lanes, Potts q = 10 52 against 64; 12 x 12, 2048
+// walkers: 40 against 40, 44 against 40), two a CTA (1280 walkers: 49 ms, with eight 56).
+static void choose_config(rewl_ctx* c, int n_sm) {
+  const Problem& P = c->P;
+  const rewl_params& prm = c->params;
+  LaunchShape s = sequential_shape(P, prm, prm.sweep_variant, n_sm);
+  if (prm.sweep_variant == kSweepChain && (prm.lanes_per_walker == 0 || prm.lanes_per_walker == 32)) {
+    const size_t limit = 227 * 1024, small = 100 * 1024;
+    const int most = c->pre_on ? 8 : kResolveWarps, asked = std::min(prm.walkers_per_block, most);
+    auto bytes = [&](int wpb) { return c->pre_on ? sweep_smem_bytes(P, wpb, 32, kSweepChain) : resolve_smem(P, wpb, false); };
+    const bool two = P.n_walkers > n_sm && bytes(2) <= small;
+    if (c->pre_on) {
+      const int wpb = asked ? asked : two ? 2 : 1;
+      if (s.G == 32 || (P.n_walkers <= 12 * n_sm && bytes(wpb) <= limit)) s = {32, wpb};
+    } else if (bytes(1) <= limit) {
+      s = {32, asked ? (bytes(asked) <= limit ? asked : 1) : two ? 2 : 1};
+    }
   }
-  c->G = G;
-  c->wpb = wpb;
+  c->G = s.G;
+  c->wpb = s.wpb;
 }
 
 // Counted copies (the e2e accounting of rewl_info.h2d_bytes / d2h_bytes).
@@ -515,9 +524,10 @@ rewl_status rewl_create(rewl_handle* out, const rewl_model* model, const rewl_la
     c->pre_buf = (PreTrial*)c->dalloc(pre_bytes, &st);
     if (st != REWL_OK) return bail(st);
   }
-  if (sweep_smem_bytes(P, charged == kSweepRing ? 1 : c->wpb, c->G, charged) > 227 * 1024)
+  const LaunchShape fits = sequential_shape(P, prm, charged, n_sm);
+  if (sweep_smem_bytes(P, fits.wpb, fits.G, charged) > 227 * 1024)
     return bail(fail(REWL_EINVAL, "a walker needs %zu bytes of shared memory (window of %d bins)",
-                     sweep_smem_bytes(P, 1, c->G, charged), P.w));
+                     sweep_smem_bytes(P, 1, fits.G, charged), P.w));
   st = upload_active(c);
   if (st != REWL_OK) return bail(st);
 #undef BAIL_CUDA

@@ -942,7 +942,6 @@ static cudaError_t launch_greedy(const Problem& P, const DevState& S, bool desce
 
 // wpb walkers a CTA, one warp each, every group of 32 trials decided together.  Bound by issue (72% of the
 // active cycles, the integer pipe 69%): 24 warps an SM at 80 registers; 64 registers for 32 warps spill and lose 6%.
-constexpr int kResolveWarps = 2;  // most walkers a CTA: they share nothing but the couplings
 template <int MODEL>
 __global__ void __launch_bounds__(32 * kResolveWarps, 12) k_sweep_resolve(Problem P, DevState S, SweepLaunch A) {
   const int first = blockIdx.x * A.wpb;
@@ -1458,11 +1457,8 @@ static cudaError_t launch_sweep_t(const Problem& P, const DevState& S, const Swe
       k_sweep_resolve_ring<MODEL><<<A.n_active, kRingThreads, ring, st>>>(P, S, A);
       return cudaGetLastError();
     }
-    SweepLaunch B = A;
-    B.wpb = std::min(A.wpb, kResolveWarps);
-    if (B.wpb > 1 && !resolve_fits(P, B.wpb)) B.wpb = 1;
-    if (resolve_fits(P, B.wpb)) {
-      k_sweep_resolve<MODEL><<<(A.n_active + B.wpb - 1) / B.wpb, B.wpb * 32, resolve_smem_bytes(P, B.wpb, false), st>>>(P, S, B);
+    if (A.wpb <= kResolveWarps && resolve_fits(P, A.wpb)) {
+      k_sweep_resolve<MODEL><<<blocks, A.wpb * 32, resolve_smem_bytes(P, A.wpb, false), st>>>(P, S, A);
       return cudaGetLastError();
     }
   }

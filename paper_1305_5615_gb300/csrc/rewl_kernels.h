@@ -23,6 +23,7 @@ cudaError_t launch_entry(const Problem& P, const DevState& S, uint64_t budget, c
 // served form (rewl_server.cu)
 int ring_walkers_per_sm(const Problem& P);
 size_t resolve_smem(const Problem& P, int wpb, bool ring);  // of the forms that decide 32 trials together
+constexpr int kResolveWarps = 2;  // most walkers a CTA of the one with own draws: they share nothing but the couplings
 size_t batch_smem_limit();  // dynamic shared memory a batched sweep CTA may use
 cudaError_t prepare_sweep_batch();
 // the walkers of d_list all belong to requests of one model (a shape group)

@@ -55,3 +55,23 @@ def test_sweeps_with_prepared_draws_take_as_long_queued_as_one_at_a_time():
     D.step(1000)
     one, queued = (t1 - t0) / 9, (D.info["sweep_ms"] - t1) / 10
     assert queued < 1.3 * one, (one, queued)
+
+
+def test_walkers_per_block_is_charged_at_the_lanes_it_was_always_charged_at():
+    """More than 8 walkers an SM with walkers per block asked for and lanes left open: accepted by the shared memory of
+    8 lanes a walker (8 x (8 B x (bins + 16) + 4 B x 128 words + 28 B x 8 trials) at L = 64), refused beyond, whatever
+    the form that runs takes; the walkers per block that are reported are those that run."""
+    m = -(-9 * n_sm() // 2)
+
+    def create(bins, wpb):
+        return rewl.REWL("ising", 64, 2, 0.75, m, 0.8, 1e-8, 5, walkers_per_block=wpb,
+                         window_starts=[0, 4097 - bins], window_widths=[bins, bins])
+
+    most = (227 * 1024 // 8 - 28 * 8 - 4 * 128) // 8 - 16
+    D = create(most, 8)
+    assert (D.info["lanes_per_walker"], D.info["walkers_per_block"], D.info["sweep_variant"]) == (32, 2, 0)
+    D.close()
+    for bins, wpb in ((most + 1, 8), (2100, 16)):     # 16 walkers of 1764 bins are the most that fit
+        with pytest.raises(rewl.RewlError) as e:
+            create(bins, wpb)
+        assert e.value.status == 1
