@@ -506,6 +506,12 @@ void rewl_server_destroy(rewl_server_handle s);
  * the window's lnf must be a power of two in [2^-39, 64].  A walker that
  * fails either is skipped (its state is left as it was) and its entry of
  * d->status, when given, is set to REWL_EINVAL; walkers that ran get 0.
+ * Calls of few walkers run the ring form, whose warps wait for one another
+ * (for microseconds).  Should such a wait last until 2^34 SM clock cycles
+ * (about 8 s) and 2^10 more for every trial have passed since the start of
+ * the launch, the walker stops part way, in the valid state of an earlier
+ * trial, with ln g and H counted up to it, and its entry is set to
+ * REWL_ETIMEOUT: do not go on from it as if all sweeps had run.
  * d->status is an optional DEVICE array of [walkers] int32 owned by the
  * caller, written on the stream like the state; with NULL the statuses are
  * not reported.
@@ -537,7 +543,8 @@ typedef struct {
   uint64_t first_sweep;                       /* sweep index of the first sweep */
   int32_t sweeps;                             /* sweeps to run (>= 0) */
   int32_t lanes_per_walker;                   /* 1, 2, 4, 8, 16 or 32; 0 = 32 */
-  int32_t* status;                            /* optional device [walkers]: 0 ran, REWL_EINVAL skipped */
+  int32_t* status;                            /* optional device [walkers]: 0 ran, REWL_EINVAL skipped,
+                                                 REWL_ETIMEOUT stopped part way */
 } rewl_sweep_desc;
 
 rewl_status rewl_sweep_noalloc(const rewl_sweep_desc* d, uint32_t* lattice, int32_t* E, double* lng, uint32_t* H,

@@ -116,9 +116,10 @@ __device__ __forceinline__ int lnf_exponent(double lnf) {
   return k;
 }
 
-// Per-walker status a sweep kernel leaves in DevState.status for a walker it
-// skipped (a walker is skipped only on inputs the library itself never makes).
-enum WalkerStatus : int32_t { kWalkerOk = 0, kWalkerBadInput = 1 };
+// Per-walker status (a rewl_status) that a sweep kernel leaves in DevState.status
+// for a walker it skipped (only on inputs the library itself never makes) or
+// stopped part way, because a wait of the ring form ran out.
+enum WalkerStatus : int32_t { kWalkerOk = 0, kWalkerBadInput = 1, kWalkerTimedOut = 4 };
 
 // Guard band of the fast acceptance test, in units of 2^-40: 2^24 units =
 // 1.5e-5 covers |logf(u) - ln u| <= 1 ulp(float) + float rounding of u

@@ -522,7 +522,7 @@ __device__ __noinline__ bool exact_accept_fx(const DevState& S, const Problem& P
 
 // ---------------------------------------------------------------------------
 // mbarriers of the ring form (rewl_resolve.cuh); every wait is bounded by a clock deadline, after which the warp
-// records an error (DevState.error) and leaves its loop.
+// records an error (DevState.error, the walker's warp also its DevState.status) and leaves its loop.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);

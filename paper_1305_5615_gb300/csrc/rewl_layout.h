@@ -70,8 +70,9 @@ struct DevState {
 
 // Sweep kernel variants (identical results): the staged form keeps H in
 // shared memory and runs a one-deep sequential chain; the chain form
-// speculates two deep and rebuilds H from the shadow; the ring form is the
-// chain form with the draws made by a second, producer warp.
+// speculates two deep and rebuilds H from the shadow (with 32 lanes that make
+// their own draws the warp decides 32 trials together instead); the ring form
+// decides 32 together, with draws made by further, producer warps.
 enum SweepVariant : int { kSweepChain = 0, kSweepStaged = 1, kSweepRing = 2 };
 
 // A trial's draw, prepared ahead of its sweep launch by k_precompute: the

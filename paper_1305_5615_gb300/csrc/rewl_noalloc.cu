@@ -24,7 +24,7 @@ namespace {
 
 // Working memory of one call, shared by all calls on a device:
 //   [0, 16)                       sweep clock (u64) and exchange round (u64)
-//   [16, 32)                      error word of the ring form's bounded waits (u32)
+//   [16, 32)                      error word of the ring form's bounded waits (u32); the walkers' statuses tell more
 //   then, each for REWL_NOALLOC_MAX_WALKERS walkers:
 //   active walker ids (i32), status flags (i32), accepted moves, near ties and
 //   exact tests (u64 each).
@@ -56,7 +56,8 @@ rewl_status scratch_address(unsigned char** out) {
 
 // Clears the part of the scratch a call uses (and the caller's status array,
 // when given: S.status points there) and fills the walker list; the sweep
-// kernel marks the walkers it skips (E outside the window, ln f not usable).
+// kernel marks the walkers it skips (E outside the window, ln f not usable)
+// and those it stops part way (a wait of the ring form ran out).
 __global__ void k_noalloc_prepare(DevState S, int n_walkers, uint64_t first_sweep) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i == 0) {
@@ -76,9 +77,15 @@ __global__ void k_noalloc_prepare(DevState S, int n_walkers, uint64_t first_swee
 
 void rewl_set_last_error(const char* msg);
 
-extern "C" rewl_status rewl_sweep_noalloc(const rewl_sweep_desc* d, uint32_t* lattice, int32_t* E, double* lng,
-                                          uint32_t* H, const uint32_t* coupling_bits, const int32_t* win_start,
-                                          const double* lnf, void* stream) {
+// The bound of the ring form's waits (SM clock cycles from the start of the launch) grows with the trials of a walker,
+// so that it is no bound on the length of a call: a trial takes 30 - 100 cycles with the GPU to itself, and one process
+// of several that share it by time slices gets a part of them while the clock goes on.
+constexpr long long kWaitCyclesPerTrial = 1 << 10;
+
+// rewl_sweep_noalloc with another constant part of that bound; for the tests.
+extern "C" rewl_status rewl_sweep_noalloc_waits(const rewl_sweep_desc* d, uint32_t* lattice, int32_t* E, double* lng,
+                                                uint32_t* H, const uint32_t* coupling_bits, const int32_t* win_start,
+                                                const double* lnf, void* stream, long long wait_cycles) {
   if (!d || !lattice || !E || !lng || !H || !win_start || !lnf) {
     rewl_set_last_error("rewl_sweep_noalloc: NULL argument");
     return REWL_EINVAL;
@@ -172,9 +179,9 @@ extern "C" rewl_status rewl_sweep_noalloc(const rewl_sweep_desc* d, uint32_t* la
   A.n_active = (int)n_walkers;
   A.wpb = wpb;
   A.variant = kSweepChain;
-  A.wait_cycles = kDefaultWaitCycles;
-  // few walkers: each one's draws by warps of their own, as rewl_create chooses; only calls that end well within the
-  // bound of that form's waits (8 s; a trial of a walker takes 20 - 100 ns)
+  A.wait_cycles = wait_cycles + (long long)A.n_att * kWaitCyclesPerTrial;
+  // few walkers: each one's draws by warps of their own, as rewl_create chooses; only calls of up to a second or two,
+  // so that the bound on their waits stays below half a minute
   int dev = 0, n_sm = 0;
   if (G == 32 && A.n_att <= (1u << 25) && cudaGetDevice(&dev) == cudaSuccess &&
       cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n_walkers <= ring_walkers_per_sm(P) * n_sm)
@@ -184,4 +191,10 @@ extern "C" rewl_status rewl_sweep_noalloc(const rewl_sweep_desc* d, uint32_t* la
     return REWL_ECUDA;
   }
   return REWL_OK;
+}
+
+extern "C" rewl_status rewl_sweep_noalloc(const rewl_sweep_desc* d, uint32_t* lattice, int32_t* E, double* lng,
+                                          uint32_t* H, const uint32_t* coupling_bits, const int32_t* win_start,
+                                          const double* lnf, void* stream) {
+  return rewl_sweep_noalloc_waits(d, lattice, E, lng, H, coupling_bits, win_start, lnf, stream, kDefaultWaitCycles);
 }

@@ -621,7 +621,10 @@ __device__ __forceinline__ void resolve_walker(const Problem& P, const DevState&
   };
 
   if constexpr (RING)
-    if (n_groups > 0 && !ring->fetch(0, lane)) return;
+    if (n_groups > 0 && !ring->fetch(0, lane)) {
+      if (lane == 0) S.status[W] = kWalkerTimedOut;
+      return;
+    }
   // A branch around code costs a lone warp about 50 cycles, leaving a loop 10 - 30: what is rare leaves the inner
   // loop, what is short is done without asking.
   for (uint32_t g = 0; g < n_groups;) {
@@ -722,7 +725,8 @@ __device__ __forceinline__ void resolve_walker(const Problem& P, const DevState&
       if (leave != 0u) break;
       commit(g);
     }
-    if (stop) {
+    if (stop) {  // told from out here: a store where the wait runs out costs the loop up to 5% (its registers)
+      if (lane == 0) S.status[W] = kWalkerTimedOut;
       add_visits(__match_any_sync(0xffffffffu, post));
       counting = 0u;
       break;
