@@ -43,7 +43,7 @@ typedef enum {
   REWL_EINVAL = 1,     /* invalid argument (see rewl_last_error) */
   REWL_ENOMEM = 2,     /* device or host allocation failed */
   REWL_ECUDA = 3,      /* a CUDA runtime call failed */
-  REWL_ETIMEOUT = 4,   /* rewl_params.timeout_ms elapsed before done */
+  REWL_ETIMEOUT = 4,   /* rewl_params.timeout_ms elapsed before done, or a kernel's bounded wait ran out */
   REWL_EENTRY = 5,     /* a walker could not reach its energy window */
   REWL_EOVERFLOW = 6,  /* a histogram counter would overflow */
   REWL_EBUSY = 7,      /* server: no capacity (request stays queued) */
@@ -122,7 +122,9 @@ typedef struct {
                                     its producer warps, in SM clock cycles from the start of a sweep
                                     launch; 0 = 2^34 (about 8 s at 2 GHz, while a launch takes
                                     milliseconds).  When a wait runs out all of them stop early and
-                                    rewl_step returns REWL_ETIMEOUT at its next flatness check */
+                                    rewl_step returns REWL_ETIMEOUT at its next flatness check.  Served
+                                    form: the request fails with REWL_ETIMEOUT; there 0 = 2^34 and 2^10
+                                    more for every trial of a walker in the launch */
   int32_t server_walker_target;  /* served form: no request is admitted while at least this many walkers of
                                     windows not yet done are running (the first always is); 0 = 24 per SM,
                                     -1 = no such limit (slots and memory only) */
@@ -452,8 +454,8 @@ typedef struct {
 
 /* device_bytes: memory budget for running requests; max_running: request slots;
  * params: sweeps_per_exchange, sweeps_per_flat_check, lnf0, entry and
- * discovery budgets and allocator of every request, server_walker_target
- * (NULL = defaults);
+ * discovery budgets, allocator and wait_cycles of every request,
+ * server_walker_target (NULL = defaults);
  * params.stream: NULL = one stream per shape group (groups overlap on the
  * device), else every group and request runs on that one stream (in order);
  * params.timeout_ms > 0: rewl_server_run fails with REWL_ETIMEOUT when no
@@ -462,7 +464,8 @@ rewl_status rewl_server_create(rewl_server_handle* out, int64_t device_bytes, in
                                const rewl_params* params);
 /* Queues a request; *id identifies it.  Errors: REWL_EINVAL (malformed),
  * REWL_ENOMEM (larger than the whole budget).  Errors found at admission
- * (e.g. REWL_EENTRY) end the request in REWL_REQ_FAILED. */
+ * (e.g. REWL_EENTRY) end the request in REWL_REQ_FAILED, and so does a
+ * bounded wait of its sweeps that runs out (REWL_ETIMEOUT; wait_cycles). */
 rewl_status rewl_server_submit(rewl_server_handle s, const rewl_request* r, uint64_t* id);
 /* Admits what fits, issues a replay of rounds for every idle group and waits
  * (without holding the server's lock) until at least one has finished;

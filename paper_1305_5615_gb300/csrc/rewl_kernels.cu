@@ -1261,7 +1261,7 @@ __global__ void __launch_bounds__(RING ? kRingThreads : 32, RING ? kBatchRingCta
   const DevState& S = slot.S;
   const uint32_t n_att = slot.n_att;
   if (!slot.active || S.done[bw.W / P.m]) return;  // uniform over the CTA
-  if constexpr (RING) sweep_resolve_ring_body<MODEL>(P, S, n_att, bw.W, kDefaultWaitCycles);
+  if constexpr (RING) sweep_resolve_ring_body<MODEL>(P, S, n_att, bw.W, slot.wait_cycles);
   else sweep_resolve_body<MODEL>(P, S, n_att, &bw.W, 1);
 }
 
@@ -1302,10 +1302,10 @@ __global__ void k_flat_batch(const BatchSlot* __restrict__ slots, int max_h) {
 __global__ void k_slot_report(const BatchSlot* __restrict__ slots, int n_slots, SlotReport* out) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= n_slots) return;
-  SlotReport r{-1, 0, 0, 0, 0};
+  SlotReport r{-1, 0, 0, 0, 0, 0};
   if (slots[s].active) {
     const uint64_t* clk = slots[s].S.clock;
-    r = SlotReport{*slots[s].S.n_done, 1, clk[0], clk[1], clk[2]};
+    r = SlotReport{*slots[s].S.n_done, 1, clk[0], clk[1], clk[2], *slots[s].S.error};
   }
   out[s] = r;
 }

@@ -87,6 +87,10 @@ struct PreTrial {
 // Default bound of the ring form's hand-off waits (SM clock cycles from the
 // start of a sweep launch): about 8 s at 2 GHz, while a launch takes milliseconds.
 constexpr long long kDefaultWaitCycles = 1ll << 34;
+// Where the caller gives no bound and none was promised, it grows with the trials of a walker, so that it is none on
+// the length of a launch: a trial takes 30 - 100 cycles with the GPU to itself, and one process of several that share
+// it by time slices gets a part of them while the clock goes on.
+constexpr long long kWaitCyclesPerTrial = 1 << 10;
 
 struct SweepLaunch {
   uint32_t n_att;     // trials per walker in this launch (sweeps * N); the first
@@ -108,6 +112,7 @@ struct BatchSlot {
   uint32_t spe;     // sweeps_per_exchange
   uint32_t spf;     // sweeps_per_flat_check
   int active;       // 0 = free slot
+  long long wait_cycles;  // bound of the ring form's hand-off waits, from the start of a launch
 };
 struct BatchWalker {
   int slot;
@@ -120,6 +125,7 @@ struct SlotReport {
   uint64_t sweeps;    // clock[0]
   uint64_t rounds;    // clock[1]
   uint64_t attempts;  // clock[2]: WL trials of all walkers (counted by the batched rounds)
+  int64_t error;      // the error word: not 0 once a wait of its ring form ran out
 };
 
 }  // namespace rewl

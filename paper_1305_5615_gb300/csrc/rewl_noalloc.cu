@@ -77,12 +77,7 @@ __global__ void k_noalloc_prepare(DevState S, int n_walkers, uint64_t first_swee
 
 void rewl_set_last_error(const char* msg);
 
-// The bound of the ring form's waits (SM clock cycles from the start of the launch) grows with the trials of a walker,
-// so that it is no bound on the length of a call: a trial takes 30 - 100 cycles with the GPU to itself, and one process
-// of several that share it by time slices gets a part of them while the clock goes on.
-constexpr long long kWaitCyclesPerTrial = 1 << 10;
-
-// rewl_sweep_noalloc with another constant part of that bound; for the tests.
+// rewl_sweep_noalloc with another constant part of its waits' bound; for the tests.
 extern "C" rewl_status rewl_sweep_noalloc_waits(const rewl_sweep_desc* d, uint32_t* lattice, int32_t* E, double* lng,
                                                 uint32_t* H, const uint32_t* coupling_bits, const int32_t* win_start,
                                                 const double* lnf, void* stream, long long wait_cycles) {

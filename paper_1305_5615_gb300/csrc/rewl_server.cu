@@ -293,6 +293,7 @@ struct rewl_server {
       b.spf = (uint32_t)h->params.sweeps_per_flat_check;
       b.n_att = b.spe * (uint32_t)h->P.N;
       b.active = 1;
+      b.wait_cycles = h->params.wait_cycles > 0 ? h->params.wait_cycles : kDefaultWaitCycles + (long long)b.n_att * kWaitCyclesPerTrial;
       g.dirty = true;
     }
     return REWL_OK;
@@ -471,6 +472,14 @@ struct rewl_server {
       r.ctx->attempts = q.attempts;
       r.ctx->n_done = q.n_done;
       r.active_walkers = (int64_t)(g.slots[s].P.h - q.n_done) * g.slots[s].P.m;
+      if (q.error != 0) {  // walkers stopped part way: its trajectory is not the request's
+        r.t_done = Clock::now();
+        r.state = REWL_REQ_FAILED;
+        r.error = REWL_ETIMEOUT;
+        ++failed;
+        release(r);
+        continue;
+      }
       if (q.n_done < g.slots[s].P.h) continue;
       r.lng.assign(r.ctx->P.n_bins, 0.0);
       const rewl_status st = rewl_get_lng(r.ctx, r.lng.data(), (int32_t)r.lng.size(), &r.n_bins, &r.e_min, &r.e_step);

@@ -431,7 +431,7 @@ class RewlServer:
 
     def __init__(self, device_bytes, max_running, sweeps_per_exchange=100, sweeps_per_flat_check=1000, lnf0=1.0,
                  entry_max_sweeps=1000, discovery_sweeps=200, stream=None, wl_rule=0, timeout_ms=0,
-                 walker_target=0):
+                 walker_target=0, wait_cycles=0):
         L = load()
         p = rewl_params_default()
         p.sweeps_per_exchange, p.sweeps_per_flat_check, p.lnf0 = sweeps_per_exchange, sweeps_per_flat_check, lnf0
@@ -439,6 +439,7 @@ class RewlServer:
         p.wl_rule = WL_RULES[wl_rule] if isinstance(wl_rule, str) else wl_rule
         p.timeout_ms = timeout_ms
         p.server_walker_target = int(walker_target)
+        p.wait_cycles = int(wait_cycles)
         if stream is not None:
             p.stream = ctypes.c_void_p(stream if isinstance(stream, int) else stream.cuda_stream)
         self._h = None
