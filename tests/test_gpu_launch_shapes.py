@@ -5,6 +5,7 @@ import numpy as np
 import pytest
 
 from paper_1305_5615_gb300 import rewl
+from parity_util import compare_states, make_pair, run_both
 
 pytestmark = pytest.mark.gpu
 
@@ -75,3 +76,14 @@ def test_walkers_per_block_is_charged_at_the_lanes_it_was_always_charged_at():
         with pytest.raises(rewl.RewlError) as e:
             create(bins, wpb)
         assert e.value.status == 1
+
+
+@pytest.mark.parametrize("prefetch", [0, 1])
+def test_windows_that_only_fit_the_sequential_chain(prefetch):
+    """24 500 bins of Potts on 256 x 256: 229 792 bytes for the chain with a whole warp, 232 864 with the tables of the
+    forms that decide 32 trials together, and a CTA has 232 448; its draws may be prepared ahead."""
+    O, D = make_pair("potts", 256, 6, 0.130016, 1, 0.8, 1e-6, 2, q=10, spe=1, spf=2, prefetch_draws=prefetch)
+    i = D.info
+    assert (i["window_bins"], i["sweep_variant"], i["lanes_per_walker"], i["prefetch_draws"]) == (24500, 0, 32, prefetch)
+    run_both(O, D, 3, 1)
+    assert compare_states(O, D, "24500 bins") == 0

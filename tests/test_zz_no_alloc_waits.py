@@ -79,3 +79,24 @@ def test_more_walkers_than_the_ring_form_runs_in_one_wave(model, q):
         torch.cuda.synchronize()
         got.append([x.cpu().numpy().view(np.uint8) for x in (lat, E, lng, H)])
     assert all(np.array_equal(a, b) for a, b in zip(*got))
+
+
+def test_a_window_that_only_fits_the_sequential_chain():
+    """28 915 bins: 232 408 bytes for the chain with a whole warp, 232 544 with the other forms' tables; a CTA has
+    232 448.  Against 8 lanes."""
+    import torch
+
+    D = rewl.REWL("ising", 16, 1, 0.75, 3, 0.8, 1e-6, 21)
+    st, bins = D.state(), 28915
+    got = []
+    for lanes in (0, 8):
+        lat, E, _, _, win, lnf = _device_state(torch, st)
+        lng = torch.zeros(3 * bins, dtype=torch.float64, device="cuda")
+        H = torch.zeros(3 * bins, dtype=torch.int32, device="cuda")
+        desc = _desc(dict(D.info, window_bins=bins), 16, 1, 3, 21, 20, lanes)
+        rewl.rewl_sweep_noalloc(desc, lat.data_ptr(), E.data_ptr(), lng.data_ptr(), H.data_ptr(), None,
+                                win.data_ptr(), lnf.data_ptr(), None)
+        torch.cuda.synchronize()
+        assert int(H.sum()) == 3 * 20 * 256
+        got.append([x.cpu().numpy().view(np.uint8) for x in (lat, E, lng, H)])
+    assert all(np.array_equal(a, b) for a, b in zip(*got))
