@@ -406,8 +406,8 @@ rewl_status rewl_thermo_jackknife(const double* lng_runs, int32_t n_runs, int32_
  * sweeps, one exchange round and, when due, the flatness check -- one fused
  * launch for the sweeps of all the group's walkers (with producer warps for
  * every walker while the GPU holds few walkers, else one warp per
- * walker), one launch each for the exchanges, clocks and flatness checks of all
- * its requests.  Every phase boundary is decided on the device (clocks,
+ * walker), one launch for the exchanges and clocks and one for the flatness
+ * checks of all its requests.  Every phase boundary is decided on the device (clocks,
  * flatness, merges and done flags are device state; the kernels of finished
  * windows and requests do nothing), so a group's k rounds and the report read
  * after them are captured once as a CUDA graph and replayed, k adapted so

@@ -940,8 +940,8 @@ static cudaError_t launch_greedy(const Problem& P, const DevState& S, bool desce
   return cudaErrorInvalidValue;
 }
 
-// wpb walkers a CTA, one warp each, every group of 32 trials decided together.  Bound by issue (72% of the
-// active cycles, the integer pipe 69%): 24 warps an SM at 80 registers; 64 registers for 32 warps spill and lose 6%.
+// wpb walkers a CTA, one warp each, every group of 32 trials decided together.  Bound by issue (69% of the
+// active cycles, the integer pipe 59% busy): 24 warps an SM at 80 registers; 64 registers for 32 warps spill and lose 6%.
 template <int MODEL>
 __global__ void __launch_bounds__(32 * kResolveWarps, 12) k_sweep_resolve(Problem P, DevState S, SweepLaunch A) {
   const int first = blockIdx.x * A.wpb;
@@ -1376,8 +1376,8 @@ cudaError_t launch_slot_report(const BatchSlot* d_slots, int n_slots, SlotReport
 constexpr size_t kMaxSmem = 227 * 1024;
 
 // Whether a whole-warp solve (32 lanes a walker, no prepared draws) runs the forms that decide 32 trials
-// together: always, unless their tables push a very wide window past the shared memory that the chain form,
-// about 1 KB smaller, still fits in.
+// together: always, unless their tables push a very wide window past the shared memory that the chain form, smaller by
+// 8 L bytes (Ising, 2D +-J), 0.5 KB + 12 L (the cube) or 1 KB + 8 L (Potts), still fits in.
 bool resolve_fits(const Problem& P, int wpb) { return resolve_smem_bytes(P, wpb, false) <= kMaxSmem; }
 size_t resolve_smem(const Problem& P, int wpb, bool ring) { return resolve_smem_bytes(P, wpb, ring); }
 

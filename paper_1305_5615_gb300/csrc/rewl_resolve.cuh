@@ -24,7 +24,7 @@
 // a trial of a walker), from ln f = 1 on 67.4 -> 47.0 ms; Potts q = 10 32 x 32, 512
 // walkers 75.1 -> 20.6 ms; +-J 12^3 114 -> 24.8 ms; Ising 8 x 8 to ln f < 1e-6
 // 615 -> 112 ms; and Ising 128 x 128, 4096 walkers, 200 sweeps 600 -> 169 - 186 ms,
-// where issue is what bounds it (385 warp instructions a group).
+// where issue is what bounds it (381 warp instructions a group).
 //
 // Visits.  ln g of a bin grows by ln f a visit, also inside the group.  For a
 // trial the counts of two bins differ by at most the number of earlier trials,

@@ -8,7 +8,7 @@
 // own: there a round is latency-bound per walker, and a fused round would make
 // every request wait for the slowest walker of all of them) --
 // one fused sweep launch over every walker of every request of the group,
-// then one launch each for the exchanges, the clocks and the due flatness
+// then one launch for the exchanges and the clocks and one for the due flatness
 // checks of all its requests.  The device decides every phase boundary: the
 // clocks, the flatness checks, the merges and the done flags live in device
 // memory and the kernels of a finished window or request do nothing, so
@@ -264,9 +264,13 @@ struct rewl_server {
         continue;
       }
       // Requests of one shape share a group (one fused launch per phase for all of them) while a
-      // round is short, i.e. launch-bound; a shape whose round lasts milliseconds (one block of
-      // N x sweeps_per_exchange trials of a walker, about 75 ns each) is latency-bound per walker,
-      // and its requests get a group each, so that no request waits for another's slowest walker.
+      // round is short, i.e. launch-bound; in a shape whose round is long (one block of
+      // N x sweeps_per_exchange trials of a walker) each walker is latency-bound, and its requests
+      // get a group each, so that no request waits for another's slowest walker.  The estimate and
+      // its line of 2 ms were set for 75 ns a trial; the forms that run now take 15 - 50 ns, so that
+      // the line lies at 0.4 - 1.3 ms.  Ising to ln f < 0.3, all requests at once, private against
+      // fused: eight of 20 x 20 258 against 271 ms, two of 32 x 32 784 against 810, but thirty-two of
+      // 20 x 20 434 against 283 and of 32 x 32 1423 against 1080.
       const double round_ms = 75e-6 * (double)h->P.N * (double)h->params.sweeps_per_exchange;
       int gi = -1;
       const rewl_status gs = group_for(r.model.kind, r.lattice.Lx, round_ms >= kPrivateRoundMs, &gi);
@@ -293,7 +297,8 @@ struct rewl_server {
       b.spf = (uint32_t)h->params.sweeps_per_flat_check;
       b.n_att = b.spe * (uint32_t)h->P.N;
       b.active = 1;
-      b.wait_cycles = h->params.wait_cycles > 0 ? h->params.wait_cycles : kDefaultWaitCycles + (long long)b.n_att * kWaitCyclesPerTrial;
+      b.wait_cycles = h->params.wait_cycles > 0 ? h->params.wait_cycles
+                                                : kDefaultWaitCycles + (long long)b.n_att * kWaitCyclesPerTrial;
       g.dirty = true;
     }
     return REWL_OK;
@@ -413,7 +418,10 @@ struct rewl_server {
     }
     if (g.n_list == 0) return REWL_OK;
     // few walkers on the GPU: each walker's passes are latency-bound, and producer warps make its
-    // draws (the ring form); many walkers share the SMs and their issue slots, and each makes its own
+    // draws (the ring form); many walkers share the SMs and their issue slots, and each makes its own.
+    // 300 and 704 walkers of Ising 16 x 16: 78 and 44 ps a trial with producer warps, 99 and 50
+    // without.  The line takes no account of windows so wide that fewer CTAs fit an SM and the ring
+    // form runs in several waves: 700 walkers of 128 x 128 (three CTAs an SM) 108 against 93.
     const bool few = active_walkers() <= kBatchRingCtas * n_sm;
     int form = kBatchChain;
     if (few && g.smem[kBatchRing] <= batch_smem_limit()) form = kBatchRing;

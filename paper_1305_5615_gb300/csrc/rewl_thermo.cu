@@ -91,7 +91,7 @@ __device__ __forceinline__ double exp_of_nonpositive(double x, const double* tab
 // centred moment (s_w holds n_bins of them, or none and they are computed again); a term of
 // exp(-746) or less, which is 0 in FP64, is not computed at all; the largest term is found
 // on the integer pipe.  rewl_thermo_jackknife of 8 runs of 1025 levels at 300 temperatures
-// (2700 CTAs) before -> after: 583 -> 348 us a call, with CUDA's exp 451.
+// (2700 CTAs) before -> after: 583 -> 348 us a call, with CUDA's exp 451; 197 since the call no longer allocates.
 constexpr uint32_t kZeroHi = 0x40875000u;  // upper word of 746
 __device__ __forceinline__ long long order_key(double v) {  // orders as the numbers do (no NaN)
   const long long i = __double_as_longlong(v);
@@ -166,7 +166,8 @@ __global__ void __launch_bounds__(256) k_thermo(const double* __restrict__ lng_t
 
 constexpr int kKeepBins = 4096;  // weights kept up to here: 32 KB of shared memory, seven CTAs an SM
 // Threads a CTA: few temperatures and tables are latency-bound, eight warps each; many fill the SMs, and then fewer
-// warps share out a table, with fewer additions across warps (that call with 256 threads 388 us, 128 353, 64 348).
+// warps share out a table, with fewer additions across warps (that call, while it allocated, with 256 threads 388 us,
+// 128 353, 64 348).
 constexpr int kFewCtas = 304;  // two an SM
 void launch_thermo(const double* tables, int n_tables, int n_bins, int e_min, int e_step, const double* T, int n_T,
                    double* out) {

@@ -40,7 +40,7 @@ extern "C" rewl_status rewl_autotune(const rewl_model* model, const rewl_lattice
     rewl_set_last_error("rewl_autotune: sweeps must be a multiple of sweeps_per_exchange");
     return REWL_EINVAL;
   }
-  // candidates: the ring form (one walker per CTA with a producer warp), and the chain form
+  // candidates: the ring form (one walker per CTA with its producer warps), and the chain form
   // with 32, 16, 8, 4 and 2 lanes per walker, walkers per CTA chosen by rewl_create
   std::vector<Candidate> cand = {{REWL_SWEEP_RING, 32, 1}, {REWL_SWEEP_CHAIN, 32, 0}, {REWL_SWEEP_CHAIN, 16, 0},
                                  {REWL_SWEEP_CHAIN, 8, 0}, {REWL_SWEEP_CHAIN, 4, 0}, {REWL_SWEEP_CHAIN, 2, 0}};
