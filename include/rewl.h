@@ -301,8 +301,9 @@ rewl_status rewl_get_state(rewl_handle h, rewl_state* st);
  * sweeps timed with CUDA events around every sweep launch.  All candidates
  * compute the same bits.  results: caller array of `capacity` entries, one per
  * candidate tried (*n_results); *best: `params` (or the defaults) with
- * sweep_variant, lanes_per_walker and walkers_per_block of the fastest, ready
- * for rewl_create.  Errors: REWL_EINVAL (arguments, sweeps not a multiple of
+ * sweep_variant, lanes_per_walker and walkers_per_block of the fastest and
+ * without prefetch_draws, as every candidate is timed, ready for rewl_create.
+ * Errors: REWL_EINVAL (arguments, sweeps not a multiple of
  * sweeps_per_exchange, no candidate ran); a candidate's own failure is in its
  * result's status.
  */

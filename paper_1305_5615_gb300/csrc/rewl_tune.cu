@@ -90,5 +90,6 @@ extern "C" rewl_status rewl_autotune(const rewl_model* model, const rewl_lattice
   best->sweep_variant = results[best_i].sweep_variant;
   best->lanes_per_walker = results[best_i].lanes_per_walker;
   best->walkers_per_block = results[best_i].walkers_per_block;
+  best->prefetch_draws = 0;  // as it was timed: with prepared draws the chain with 32 lanes is another form
   return REWL_OK;
 }

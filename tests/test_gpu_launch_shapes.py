@@ -1,6 +1,8 @@
 """Which form a solve runs in and with which launch shape, where an option or a
 forced shape meets the automatic choice; the states are the same bits in every
 form."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -87,3 +89,21 @@ def test_windows_that_only_fit_the_sequential_chain(prefetch):
     assert (i["window_bins"], i["sweep_variant"], i["lanes_per_walker"], i["prefetch_draws"]) == (24500, 0, 32, prefetch)
     run_both(O, D, 3, 1)
     assert compare_states(O, D, "24500 bins") == 0
+
+
+def test_autotune_returns_what_it_timed():
+    """The candidates are timed without prepared draws, so the best is returned without them: 9 walkers an SM take the
+    chain with a whole warp, which with them is the sequential form."""
+    m = -(-9 * n_sm() // 4)
+    p, best = rewl.rewl_params_default(), rewl.rewl_params()
+    p.sweeps_per_exchange, p.sweeps_per_flat_check, p.prefetch_draws = 20, 100, 1
+    res, n = (rewl.rewl_tune_result * 8)(), ctypes.c_int32()
+    args = (rewl.rewl_model(0, 2), rewl.rewl_lattice(2, 8, 8, 1))
+    assert rewl.load().rewl_autotune(ctypes.byref(args[0]), ctypes.byref(args[1]), None, 4, 0.75, m, 0.8, 1e-8,
+                                     ctypes.c_uint64(5), ctypes.byref(p), 40, res, 8, ctypes.byref(n),
+                                     ctypes.byref(best)) == 0
+    h = rewl.rewl_create(*args, None, 4, 0.75, m, 0.8, 1e-8, 5, best)
+    i = rewl.rewl_get_info(h)
+    rewl.rewl_destroy(h)
+    assert i["prefetch_draws"] == 0
+    assert (i["sweep_variant"], i["lanes_per_walker"]) == (best.sweep_variant, best.lanes_per_walker)
